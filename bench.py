@@ -36,10 +36,14 @@ STEP_KERNELS = {1: ("step_kernel (one-step: fused AA collide-stream-QoI, in plac
                     "collided again, pushed to the other lattice)", "step2_kernel", "two-step-v2-packed"),
                 4: ("strip2_kernel (two-step row strips: each row collided into a shared-memory ring, streamed "
                     "and collided again, pushed to the other lattice)", "strip2_kernel", "two-step-strips-v2-staged"),
-                6: ("strip3w_kernel (three-step row strips at a compile-time width: each row collided into a "
-                    "first shared-memory ring, streamed and collided into a second, streamed and collided again, "
-                    "pushed to the other lattice)", "strip3w_kernel", "three-step-strips-fixed-width-v3")}
-STEPS_PER_LAUNCH = {1: 1, 3: 2, 4: 2, 6: 3, 7: 1}
+                6: ("strip_regs_kernel (row strips with three or four steps per launch: each warp walks a window of "
+                    "64 columns down its rows and keeps the rows between the steps in registers)", "strip_regs_kernel",
+                    "strips-in-registers-v1")}
+
+
+def steps_per_launch_of(scheme: int, storage: str) -> int:
+    """Time steps one launch of the scheme's kernel advances (the register strips: four in FP32)."""
+    return {1: 1, 3: 2, 4: 2, 6: 4 if storage == "f32" else 3, 7: 1}.get(scheme, 1)
 
 
 def _traffic_file(kernel: str, storage: str) -> str:
@@ -258,7 +262,7 @@ def bench_kernel_only(args):
     torch.cuda.synchronize()
     ms, st, la = U.uqlb_last_loop_time(ens.ctx)
     scheme, g_rows, g_npt = U.uqlb_last_run_geometry(ens.ctx)
-    per_launch = STEPS_PER_LAUNCH.get(scheme, 1)
+    per_launch = steps_per_launch_of(scheme, args.storage)
     nodes = sum(s.nx * s.ny for s in smp)
     gbs = BYTES_PER_UPDATE[args.storage] * nodes / (ms / max(st / per_launch, 1) / 1e3) / 1e9
     print(json.dumps({"kernel_only": True, "mode": args.mode, "scheme": scheme, "tile": [g_rows, g_npt],
@@ -273,8 +277,8 @@ def bench_kernel_only(args):
 
 def tune_summary(tuned):
     """The autotuner's candidates as labels with their ms per step: tile geometries "rows x npt", and on
-    the three-step strips "<staging>/<blocks per SM>b/<shared-memory KB>k" (staging "s0": none, "s1": one
-    row in shared memory, "r1": one row in registers, "g": the generic-width kernel)."""
+    the three-step strips "<staging>/<blocks per SM>b/<shared-memory KB>k" (staging "s0": none, "s1": the
+    next rows in shared memory, "r1": one row in registers, "g": the generic-width kernel)."""
     if tuned is None:
         return None
 
@@ -720,7 +724,7 @@ def bench_gpu(args):
     # roofline of the dominant kernel, from its event-timed loop.  One launch reads and writes
     # every population once (72 B per FP32 node); the two-step kernel advances two steps per launch.
     scheme, g_rows, g_npt = U.uqlb_last_run_geometry(ens.ctx)
-    steps_per_launch = STEPS_PER_LAUNCH[scheme]
+    steps_per_launch = steps_per_launch_of(scheme, storage)
     kernel_name, ncu_name, kernel_version = STEP_KERNELS[scheme]
     nodes = (hi - lo) * w.base.nx * w.base.ny
     per_launch_bytes = BYTES_PER_UPDATE[storage] * nodes

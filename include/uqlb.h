@@ -195,12 +195,11 @@ typedef struct {
     int32_t scheme;           /* time-stepping scheme, UQLB_SCHEME_* (see below) */
     /* Launch shape of the three-step row strips (ignored by the other kernels); each 0: the value
      * the context's autotuner picked for this batch shape, else the default. */
-    int32_t strip_blocks_per_sm; /* resident blocks per SM (at most what fits; the grid is
-                                    min(rows, blocks per SM x SMs) and each block takes an equal
-                                    share of the rows) */
+    int32_t strip_blocks_per_sm; /* resident blocks of 128 threads per SM (at most what fits; their warps
+                                    take equal shares of the rows) */
     int32_t strip_stage;      /* widths 64, 128, 256, 512, 1024: 1 = rows not staged, 2 = the next
-                                 row staged in shared memory by cp.async, 3 = the next row loaded
-                                 into registers (other widths: 0 only) */
+                                 three rows staged in shared memory by cp.async, 3 = the next row
+                                 loaded into registers (other widths: 0 only) */
     int32_t strip_smem_kb;    /* shared-memory share per SM in KB: 8, 16, 32, 64, 100, 132, 164, 196
                                  or 228 (the rest of the 256 KB is L1); raised to what the blocks
                                  per SM need */
@@ -226,12 +225,12 @@ typedef struct {
  *       TWO_STEP_TILES: blocks take tiles of the tile geometry with a one-node halo (any size,
  *         FP64 too; the halo is collided twice, 27 % more collisions at tile 8 x 128).
  *     UQLB_SCHEME_TWO_STEP takes strips where the batch allows them, else tiles.
- *   UQLB_SCHEME_THREE_STEP_STRIPS: one launch per three time steps on the row strips, two rings of
- *     collided rows in shared memory (24 B of HBM traffic per FP32 node update); widths up to 1600
- *     (1280 with FP32 storage), the same storage formats and lattices as TWO_STEP_STRIPS.  A sample
- *     with fewer than three steps left runs two or one in its last launch.  With FP32 storage its
- *     fields equal the two-step strips' bit for bit (the same packed collisions of the same node
- *     pairs; FP32 rows pass through shared memory and HBM unrounded).
+ *   UQLB_SCHEME_THREE_STEP_STRIPS: one launch per three time steps (16-bit storage; 12 B of HBM traffic
+ *     per node update) or four (FP32 storage, whose rows pass unrounded between launches; 18 B) on the row
+ *     strips, the rows between the steps in registers; widths up to 1600 (1280 with FP32 storage), the
+ *     same storage formats and lattices as TWO_STEP_STRIPS.  A sample with fewer steps left runs those in
+ *     its last launch.  With FP32 storage its fields equal the two-step strips' bit for bit (the same
+ *     packed collisions; FP32 rows pass between steps and through HBM unrounded).
  *   UQLB_SCHEME_CLUSTER: CHANNEL samples with the halfway obstacle and the face inlet/outlet, FP32
  *     or 16-bit storage, UQLB_MODE_GRAPH: one thread-block cluster per sample holds the sample's
  *     lattice in shared memory (split into slabs of columns over up to 16 blocks, one copy, updated
@@ -243,10 +242,10 @@ typedef struct {
  *     run at once.  Fields equal the one-step scheme's bit for bit; C_D and C_L sum the same link
  *     forces in another order (FP32 round-off).  One workspace lattice, as ONE_STEP.
  *   UQLB_SCHEME_AUTO: the row strips for periodic FP32, FP16, BF16 and FX16 batches in graph mode,
- *     three steps per launch where the width allows it, else two, else TWO_STEP_TILES (measured on
- *     GB300, 625 x 256^2 ensemble, kernel GLUPS three-step strips / two-step strips / tiles /
- *     one-step: FP32 242 / 179 / 115 / 84, BF16 234 / 184 / 103 / 90, FP16 231 / 173 / 95 / 82,
- *     FX16 216 / 170 / - / -); CLUSTER for CHANNEL batches that allow it (FP32 9 x 440 x 82 cylinder
+ *     three or four steps per launch where the width allows it, else two, else TWO_STEP_TILES (measured
+ *     on GB300, 625 x 256^2 ensemble, kernel GLUPS three-step strips / two-step strips / tiles /
+ *     one-step: FP32 324 / 179 / 115 / 84, BF16 294 / 184 / 103 / 90, FP16 280 / 173 / 95 / 82,
+ *     FX16 227 / 170 / - / -); CLUSTER for CHANNEL batches that allow it (FP32 9 x 440 x 82 cylinder
  *     samples: 60 against 24 GLUPS on ONE_STEP); ONE_STEP otherwise (FP64 is bound by the FP64
  *     rate).  In graph mode with FP32/FP16/BF16/FX16 storage a batch of unlike samples runs as
  *     groups of like samples, each on its own kernel and its own slice of the workspace
@@ -261,7 +260,7 @@ typedef struct {
  *     caller's rows.
  *     uqlb_last_run_geometry then reports UQLB_SCHEME_GROUPED.
  * A resumed run (start_step > 0) continues the state on any multi-step kernel (the strips and the
- * tiles, with two or three steps per launch, leave the same lattice layout); a one-step run resumes
+ * tiles, with two to four steps per launch, leave the same lattice layout); a one-step run resumes
  * on the one-step scheme only, a cluster run on the cluster scheme (it leaves the natural layout). */
 enum {
     UQLB_SCHEME_AUTO = 0,
@@ -388,7 +387,7 @@ int uqlb_batch_workspace_bytes(const uqlb_sample* samples, int64_t n, const uqlb
 /* Run n independent samples on the device: initialise every lattice at equilibrium, step all
  * samples with the collision, streaming, boundaries and QoI reductions fused into the step kernels
  * of the run's scheme (uqlb_run_opts.scheme: in place in AA order with one launch per step, or two
- * lattices with two or three steps per launch; under UQLB_SCHEME_AUTO periodic FP32/16-bit batches
+ * lattices with two to four steps per launch; under UQLB_SCHEME_AUTO periodic FP32/16-bit batches
  * take two lattices, so size the workspace with uqlb_batch_workspace_bytes for the same options),
  * and write the results.
  *   workspace_dev / workspace_bytes: scratch of at least uqlb_batch_workspace_bytes bytes,

@@ -249,6 +249,11 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
     return d;
 }
 __device__ __forceinline__ f2 splat(float c) { return pk(c, c); }
+__device__ __forceinline__ float rcp_approx(float v) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
 
 // Relaxation constants of the packed collision for one relaxation rate omega.  The BGK update is
 // written as g_i* = (1 - omega) g_i + omega g_i^eq, with omega folded into the equilibrium's
@@ -288,12 +293,13 @@ __device__ __forceinline__ void collide_packed(f2 (&g)[9], const PackedBGK& k, f
     const f2 a = sub2(g[5], g[7]), b = sub2(g[6], g[8]);
     const f2 jx = add2(sub2(g[1], g[3]), sub2(a, b));
     const f2 jy = add2(sub2(g[2], g[4]), add2(a, b));
-    float da, db;
-    upk(drho, da, db);
-    // 1/rho - 1 per node; the fast division (reciprocal and multiply, within 2 ulp) is exact enough
-    // for this small correction (|drho| << 1: its error is ~1e-7 of ~1e-4 of u) and saves the
-    // IEEE division's refinement steps
-    const f2 d = pk(__fdividef(-da, 1.0f + da), __fdividef(-db, 1.0f + db));
+    // d = 1/rho - 1 = drho * (1 / -(1 + drho)) per node: the approximate reciprocal (1 ulp) is exact
+    // enough for this small correction (|drho| << 1: its error is ~1e-7 of ~1e-4 of u).  The same bits as
+    // __fdividef(-drho, 1 + drho) (rounding is symmetric in the sign), whose range checks of the divisor
+    // took a third of the strips' non-FMA instructions.
+    float ra, rb;
+    upk(sub2(splat(-1.0f), drho), ra, rb);
+    const f2 d = mul2(drho, pk(rcp_approx(ra), rcp_approx(rb)));
     const f2 ux = fma2(jx, d, jx), uy = fma2(jy, d, jy);
     if (usq != nullptr) *usq = fma2(uy, uy, mul2(ux, ux));
     const f2 X = fma2(splat(-1.5f), fma2(jy, uy, mul2(jx, ux)), drho);
@@ -323,6 +329,42 @@ __device__ __forceinline__ void collide_packed(f2 (&g)[9], const PackedBGK& k, f
         g[i] = fma2(g[i], k.omc, fma2(ol, cj, oA));
         g[o] = fma2(g[o], k.omc, fma2(nl, cj, oA));
     }
+}
+
+// One half of collide_packed() in scalar FP32: the same operations in the same order, so the same bits.
+__device__ __forceinline__ void collide_half(float (&g)[9], const PackedBGK& k) {
+    const float omc = __uint_as_float((uint32_t)k.omc), ow0 = __uint_as_float((uint32_t)k.ow0),
+                ow1 = __uint_as_float((uint32_t)k.ow1), ow5 = __uint_as_float((uint32_t)k.ow5),
+                ol1 = __uint_as_float((uint32_t)k.ol1), ol5 = __uint_as_float((uint32_t)k.ol5);
+    const float drho = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(g[0], g[1]), __fadd_rn(g[2], g[3])),
+                                           __fadd_rn(__fadd_rn(g[4], g[5]), __fadd_rn(g[6], g[7]))), g[8]);
+    const float a = __fsub_rn(g[5], g[7]), b = __fsub_rn(g[6], g[8]);
+    const float jx = __fadd_rn(__fsub_rn(g[1], g[3]), __fsub_rn(a, b));
+    const float jy = __fadd_rn(__fsub_rn(g[2], g[4]), __fadd_rn(a, b));
+    const float d = __fmul_rn(drho, rcp_approx(__fsub_rn(-1.0f, drho)));
+    const float ux = __fmaf_rn(jx, d, jx), uy = __fmaf_rn(jy, d, jy);
+    const float X = __fmaf_rn(-1.5f, __fmaf_rn(jy, uy, __fmul_rn(jx, ux)), drho);
+    const float ux45 = __fmul_rn(4.5f, ux), uy45 = __fmul_rn(4.5f, uy);
+    g[0] = __fmaf_rn(g[0], omc, __fmul_rn(ow0, X));
+#pragma unroll
+    for (int i : {1, 2, 5, 6}) {
+        const int o = opp(i);
+        const float cj = i == 1 ? jx : (i == 2 ? jy : (i == 5 ? __fadd_rn(jx, jy) : __fsub_rn(jy, jx)));
+        const float cu = i == 1 ? ux45 : (i == 2 ? uy45 : (i == 5 ? __fadd_rn(ux45, uy45) : __fsub_rn(uy45, ux45)));
+        const float ow = i <= 4 ? ow1 : ow5, ol = i <= 4 ? ol1 : ol5;
+        const float oA = __fmul_rn(ow, __fmaf_rn(cj, cu, X));
+        g[i] = __fmaf_rn(g[i], omc, __fmaf_rn(ol, cj, oA));
+        g[o] = __fmaf_rn(g[o], omc, __fmaf_rn(-ol, cj, oA));
+    }
+}
+__device__ __forceinline__ void collide_halves(f2 (&g)[9], const PackedBGK& k) {
+    float a[9], b[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) upk(g[i], a[i], b[i]);
+    collide_half(a, k);
+    collide_half(b, k);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = pk(a[i], b[i]);
 }
 
 // collide_packed() on two nodes held as separate arrays.

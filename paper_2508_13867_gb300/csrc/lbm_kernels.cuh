@@ -12,7 +12,7 @@
 // to slot opp(i)); an odd step reads the incoming populations from the neighbours' slots and
 // writes its outgoing populations into the neighbours' slots.  Every memory location is read and
 // then written by exactly one thread per step, so no second lattice and no intra-step
-// synchronisation are needed.  Multi-step schemes (periodic batches; strip2_kernel and strip3_kernel
+// synchronisation are needed.  Multi-step schemes (periodic batches; strip2_kernel and strip_regs_kernel
 // on row strips, step2_kernel on tiles): two lattices in natural order, each launch collides,
 // streams through shared memory, collides again (once or twice) and pushes into the other lattice.
 // Boundary rules are applied where a population crosses a boundary link:
@@ -1419,726 +1419,7 @@ __global__ void __launch_bounds__(1024, 1) strip2_kernel(KParams p) {
     }
 }
 
-// ------------------------------------------------------------------------------------------
-// Three steps per launch by row strips (periodic batches of one width).
-// ------------------------------------------------------------------------------------------
-// The same walk as strip2_kernel with one more collision per node: for row y of its range a block
-// collides row y + 2 at step t into ring 1 (phase A), waits, gathers row y + 1 of step t + 1 from
-// rows y .. y + 2 of ring 1, collides it into ring 2 (phase B), waits, then gathers row y of step
-// t + 2 from rows y - 1 .. y + 1 of ring 2, collides it and pushes it into the other lattice
-// (phase C).  Each piece (the rows of one sample in one block's range) starts with four extra
-// phase-A rows and two extra phase-B rows, so a launch collides (3L + 6) / 3L nodes per node of an
-// L-row piece and moves every population through HBM once per three steps (24 B per FP32 node
-// update against 36 B with two steps per launch).  A sample with fewer than three steps left runs
-// two (phases A and B, B pushing) or one (collide and push) in its last launch.
-//
-// Rings: population i of a row is read by the next phase at row y + c_iy.  With two barriers per
-// iteration, every read of a ring precedes (through a barrier) the next iteration's writes to it, so
-// the c_iy = +1 group needs 3 slots, c_iy = 0 two and c_iy = -1 one: 6 slots of 3 planes per ring.
-constexpr int kRing3Planes = 18;
-
-// Plane of direction i for the row with index q (q >= 0: rows counted from a fixed origin below the
-// piece) in a ring of 3 / 2 / 1 slots per group.
-__device__ __forceinline__ int ring3_plane(int i, int q) {
-    switch (i) {
-        case 2: return (q % 3) * 3 + 0;
-        case 5: return (q % 3) * 3 + 1;
-        case 6: return (q % 3) * 3 + 2;
-        case 0: return 9 + (q & 1) * 3 + 0;
-        case 1: return 9 + (q & 1) * 3 + 1;
-        case 3: return 9 + (q & 1) * 3 + 2;
-        case 4: return 15;
-        case 7: return 16;
-        default: return 17;
-    }
-}
-
-// Tuning of the three-step strips (as for the two-step strips: staged phase-A rows and the
-// shared-memory share per SM; 0 = the largest), and the form of its collisions: packed pairs (0) or
-// two scalar collisions per pair (1; FP32 pipe instead of the packed pipe).
-#ifndef UQLB_STRIP3_PREFETCH_F32
-#define UQLB_STRIP3_PREFETCH_F32 UQLB_STRIP_PREFETCH_F32
-#endif
-#ifndef UQLB_STRIP3_PREFETCH_16
-#define UQLB_STRIP3_PREFETCH_16 UQLB_STRIP_PREFETCH_16
-#endif
-#ifndef UQLB_STRIP3_CARVEOUT_F32_KB
-#define UQLB_STRIP3_CARVEOUT_F32_KB UQLB_STRIP_CARVEOUT_F32_KB
-#endif
-#ifndef UQLB_STRIP3_CARVEOUT_16_KB
-#define UQLB_STRIP3_CARVEOUT_16_KB UQLB_STRIP_CARVEOUT_16_KB
-#endif
-#ifndef UQLB_STRIP3_COLLIDE
-#define UQLB_STRIP3_COLLIDE 0
-#endif
-__device__ __forceinline__ void strip3_collide(f2 (&g)[9], float omega, const PackedBGK& omega2, f2* usq) {
-    if constexpr (UQLB_STRIP3_COLLIDE == 0) {
-        collide_packed(g, omega2, usq);
-    } else {
-        float a[9], b[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) upk(g[i], a[i], b[i]);
-        float qa = 0.0f, qb = 0.0f;
-        collide_pair_scalar(a, b, omega, usq != nullptr ? &qa : nullptr, usq != nullptr ? &qb : nullptr);
-        if (usq != nullptr) *usq = pk(qa, qb);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) g[i] = pk(a[i], b[i]);
-    }
-}
-
-template <typename S>
-struct Strip3Tune {
-    static constexpr int depth = sizeof(S) == 4 ? UQLB_STRIP3_PREFETCH_F32 : UQLB_STRIP3_PREFETCH_16;
-    static constexpr int carveout_kb = sizeof(S) == 4 ? UQLB_STRIP3_CARVEOUT_F32_KB : UQLB_STRIP3_CARVEOUT_16_KB;
-    static constexpr int max_nx_raw = (232448 - 2048) / (2 * kRing3Planes * 4 + depth * 9 * (int)sizeof(S)) / 64 * 64;
-    static constexpr int max_nx = max_nx_raw < 2048 ? max_nx_raw : 2048;
-};
-
-template <typename S, bool GENERIC>
-__global__ void __launch_bounds__(1024, 1) strip3_kernel(KParams p) {
-    extern __shared__ __align__(16) unsigned char s4_raw[];
-    __shared__ __align__(16) SampleDev s_sp;
-    __shared__ int s_j, s_rows, s_nact, s_flag;
-    const int tid = threadIdx.x, np = blockDim.x;
-    const int rw = 2 * np;
-    float* ring1 = reinterpret_cast<float*>(s4_raw);  // [kRing3Planes][rw]
-    float* ring2 = ring1 + kRing3Planes * rw;         // [kRing3Planes][rw]
-    double* s_red = reinterpret_cast<double*>(s4_raw);  // block sums: the rings, once a piece is done
-    S* stage = reinterpret_cast<S*>(ring2 + kRing3Planes * rw);  // [D][9][rw]
-    const int t = (int)p.step_counter[0] + p.dt;
-    const int t0 = (int)p.step_counter[1];
-    if (tid == 0) {
-        const int nact = active_samples(p, t);
-        s_nact = nact;
-        s_rows = p.row_base[nact];
-    }
-    __syncthreads();
-    const int nact = s_nact, rows = s_rows;
-    const int per = (rows + gridDim.x - 1) / gridDim.x;
-    const int r0 = blockIdx.x * per, r1 = min(rows, r0 + per);
-    const bool series = p.qoi_every > 0 && p.series != nullptr;
-    const bool sr = sizeof(S) == 2 && p.stochastic != 0;
-    const int nx = GENERIC ? __ldg(&p.samples[0].nx) : rw;
-    const int x = 2 * tid;
-    const bool va = !GENERIC || x < nx, vb = !GENERIC || x + 1 < nx;
-    const int xl = x == 0 ? nx - 1 : x - 1;
-    const int xar = GENERIC && x + 1 >= nx ? x + 1 - nx : x + 1;
-    const int xbr = x + 2 >= nx ? x + 2 - nx : x + 2;
-    constexpr int D = Strip3Tune<S>::depth;
-    for (int r = r0; r < r1;) {
-        __syncthreads();  // the previous piece's ring reads and block sums are done
-        if (tid == 0) {
-            int lo = 0, hi = nact - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (p.row_base[mid] <= r)
-                    lo = mid;
-                else
-                    hi = mid - 1;
-            }
-            s_j = lo;
-        }
-        __syncthreads();
-        const int j = s_j;
-        if (tid < 32) reinterpret_cast<uint32_t*>(&s_sp)[tid] = __ldg(reinterpret_cast<const uint32_t*>(p.samples + j) + tid);
-        __syncthreads();
-        const int rb = p.row_base[j];
-        const int ny = s_sp.ny, pitch = s_sp.pitch, plane = (int)s_sp.plane;
-        const int ya = r - rb, yb = min(ny, r1 - rb);
-        r = rb + yb;
-        const int n = min(3, s_sp.steps - t);  // steps of this launch for this sample (>= 1)
-        bool want[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) want[k] = series && k < n && ((t + k) % p.qoi_every) == 0;
-        const bool second = ((p.sel[s_sp.slot] ^ ((t - t0) / 3)) & 1) != 0;
-        const S* src = static_cast<const S*>(second ? p.arena2 : p.arena) + s_sp.f_off;
-        S* dst = static_cast<S*>(second ? p.arena : p.arena2) + s_sp.f_off;
-        const float omega = (float)s_sp.omega;
-        const PackedBGK omega2 = packed_bgk(omega);
-        const uint32_t sid = (uint32_t)s_sp.sample_id;
-        const typename Storage<S>::Q qz = quanta_of<S>(p, j);
-        double red[3] = {0.0, 0.0, 0.0};
-        // periodic row of a phase-A row (at most two rows outside the sample; samples have >= 2 rows,
-        // two corrections each way keep any height in range)
-        auto wrap = [&](int y) {
-            y += y < 0 ? ny : 0;
-            y += y < 0 ? ny : 0;
-            y -= y >= ny ? ny : 0;
-            y -= y >= ny ? ny : 0;
-            return y;
-        };
-        // push of the pair's post-collision populations g (step ts, row y) into dst
-        auto push = [&](int y, int ts, const f2 (&g)[9]) {
-            const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
-            const int row[3] = {ym * pitch, y * pitch, yp * pitch};
-            if constexpr (sizeof(S) == 2) {
-                // 16-bit storage: each population's pair rounded into one word (one hash per pair and
-                // step for the stochastic bits), stored whole where it stays in its columns
-                uint32_t h = 0u;
-                if (sr)
-                    h = mix32((uint32_t)(y * pitch + x) * 0x9E3779B1u + (uint32_t)ts * 0x85EBCA77u +
-                              sid * 0xC2B2AE3Du);
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    S* d = dst + (i * plane + row[1 + cy(i)]);
-                    const uint32_t w =
-                        sr ? pair_word_sr<S>(g[i], sr_bits(h, i), qz, i) : pair_word<S>(g[i], qz, i);
-                    if (cx(i) == 0 && vb) {
-                        *reinterpret_cast<uint32_t*>(d + x) = w;
-                    } else {
-                        const int ca = cx(i) == 0 ? x : (cx(i) > 0 ? xar : xl);
-                        const int cb = cx(i) == 0 ? x + 1 : (cx(i) > 0 ? xbr : x);
-                        *reinterpret_cast<uint16_t*>(d + ca) = (uint16_t)w;
-                        if (vb) *reinterpret_cast<uint16_t*>(d + cb) = (uint16_t)(w >> 16);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    S* d = dst + (i * plane + row[1 + cy(i)]);
-                    float a, b;
-                    upk(g[i], a, b);
-                    const int ca = cx(i) == 0 ? x : (cx(i) > 0 ? xar : xl);
-                    const int cb = cx(i) == 0 ? x + 1 : (cx(i) > 0 ? xbr : x);
-                    if (cx(i) == 0 && vb) {
-                        pair_store<S>(d + x, g[i], qz, i);
-                    } else {
-                        Storage<S>::store(d + ca, a, qz, i);
-                        if (vb) Storage<S>::store(d + cb, b, qz, i);
-                    }
-                }
-            }
-        };
-        auto add_usq = [&](double& acc, f2 q) {
-            float a, b;
-            upk(q, a, b);
-            acc += (double)a;
-            if (vb) acc += (double)b;
-        };
-        // gather of row y's pair from a ring (population i from ring row y - c_iy, column x - c_ix);
-        // oq: ring row index of row y (rows y - 1 and y + 1 are oq - 1 and oq + 1)
-        auto gather = [&](const float* ring, int oq, f2 (&g)[9]) {
-            const float* rp = ring + ring3_plane(2, oq - 1) * rw;  // c_iy = +1: row y - 1 (planes 2, 5, 6)
-            const float* rz = ring + ring3_plane(0, oq) * rw;      // c_iy =  0: row y     (planes 0, 1, 3)
-            const float* rm = ring + ring3_plane(4, oq + 1) * rw;  // c_iy = -1: row y + 1 (planes 4, 7, 8)
-            g[0] = *reinterpret_cast<const f2*>(rz + x);
-            g[1] = pk(rz[rw + xl], rz[rw + x]);
-            g[3] = pk(rz[2 * rw + xar], rz[2 * rw + xbr]);
-            g[2] = *reinterpret_cast<const f2*>(rp + x);
-            g[5] = pk(rp[rw + xl], rp[rw + x]);
-            g[6] = pk(rp[2 * rw + xar], rp[2 * rw + xbr]);
-            g[4] = *reinterpret_cast<const f2*>(rm + x);
-            g[7] = pk(rm[rw + xar], rm[rw + xbr]);
-            g[8] = pk(rm[2 * rw + xl], rm[2 * rw + x]);
-        };
-        auto put_ring = [&](float* ring, int oq, const f2 (&g)[9]) {
-            f2* r2 = reinterpret_cast<f2*>(ring);
-#pragma unroll
-            for (int i = 0; i < 9; ++i) r2[ring3_plane(i, oq) * np + tid] = g[i];
-        };
-        if (n == 1) {
-            // the sample's last step: collide and push row by row
-            for (int y = ya; y < yb && va; ++y) {
-                const S* s0 = src + (y * pitch + x);
-                f2 g[9];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) g[i] = pair_load<S>(s0 + i * plane, qz, i);
-                f2 q;
-                strip3_collide(g, omega, omega2, want[0] ? &q : nullptr);
-                if (want[0]) add_usq(red[0], q);
-                push(y, t, g);
-            }
-        } else {
-            // phase-A rows run from ya - (n == 3 ? 2 : 1) to yb + n - 2; ring row index of row y:
-            // y - ya + 4 (>= 0 for every row the piece touches)
-            const int a0 = ya - (n - 1);
-            auto fetch = [&](int qa) {
-                // staging: phase-A row a0 + qa goes to buffer qa % D, D rows ahead of its phase A; one
-                // copy group per row (empty past the piece)
-                if (va && a0 + qa <= yb + n - 2) {
-                    const S* s0 = src + (wrap(a0 + qa) * pitch + x);
-                    S* st = stage + (qa % (D > 0 ? D : 1)) * 9 * rw + x;
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) cp_async<2 * sizeof(S)>(st + i * rw, s0 + i * plane);
-                }
-                cp_async_commit();
-            };
-            (void)fetch;
-            auto phase_a = [&](int ya_row) {
-                if (!va) return;
-                const int qa = ya_row - a0;
-                f2 g[9];
-                if constexpr (D > 0) {
-                    cp_async_wait<D - 1>();
-                    const S* st = stage + (qa % D) * 9 * rw + x;
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) g[i] = pair_load<S>(st + i * rw, qz, i);
-                    fetch(qa + D);
-                } else {
-                    const S* s0 = src + (wrap(ya_row) * pitch + x);
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) g[i] = pair_load<S>(s0 + i * plane, qz, i);
-                }
-                f2 qq;
-                const bool w = want[0] && ya_row >= ya && ya_row < yb;
-                strip3_collide(g, omega, omega2, w ? &qq : nullptr);
-                if (w) add_usq(red[0], qq);
-                put_ring(ring1, ya_row - ya + 4, g);
-            };
-#pragma unroll
-            for (int k = 0; k < D; ++k) fetch(k);
-            if (n == 3) {
-                phase_a(ya - 2);
-                phase_a(ya - 1);
-                for (int y = ya - 2; y < yb; ++y) {
-                    phase_a(y + 2);
-                    __syncthreads();
-                    if (va) {
-                        // phase B: row y + 1 at step t + 1 from ring 1, into ring 2
-                        f2 g[9];
-                        gather(ring1, y + 1 - ya + 4, g);
-                        f2 qq;
-                        const bool w = want[1] && y + 1 >= ya && y + 1 < yb;
-                        strip3_collide(g, omega, omega2, w ? &qq : nullptr);
-                        if (w) add_usq(red[1], qq);
-                        put_ring(ring2, y + 1 - ya + 4, g);
-                    }
-                    __syncthreads();
-                    if (va && y >= ya) {
-                        // phase C: row y at step t + 2 from ring 2, pushed into the other lattice
-                        f2 g[9];
-                        gather(ring2, y - ya + 4, g);
-                        f2 qq;
-                        strip3_collide(g, omega, omega2, want[2] ? &qq : nullptr);
-                        if (want[2]) add_usq(red[2], qq);
-                        push(y, t + 2, g);
-                    }
-                }
-            } else {
-                phase_a(ya - 1);
-                for (int y = ya - 1; y < yb; ++y) {
-                    phase_a(y + 1);
-                    __syncthreads();
-                    if (va && y >= ya) {
-                        // phase B: row y at step t + 1 from ring 1, pushed into the other lattice
-                        f2 g[9];
-                        gather(ring1, y - ya + 4, g);
-                        f2 qq;
-                        strip3_collide(g, omega, omega2, want[1] ? &qq : nullptr);
-                        if (want[1]) add_usq(red[1], qq);
-                        push(y, t + 1, g);
-                    }
-                    __syncthreads();
-                }
-            }
-            if constexpr (D > 0) cp_async_wait<0>();  // the empty groups past the piece
-        }
-        if (want[0] || want[1] || want[2]) {
-            // this piece's sums; the block that completes the sample adds the pieces in row order
-            __syncthreads();  // s_red lives in the rings
-            block_sum_dyn<3>(red, s_red);
-            if (tid == 0) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) p.partials[(int64_t)(rb + ya) * 3 + k] = red[k];
-                __threadfence();
-                const int prev = atomicAdd(p.counters + j, yb - ya);
-                s_flag = (prev + (yb - ya) == ny);
-            }
-            __syncthreads();
-            if (s_flag) {
-                __threadfence();
-                double acc[3] = {0.0, 0.0, 0.0};
-                for (int q = tid; q < ny; q += np) {
-                    if (q == 0 || (rb + q) % per == 0) {
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) acc[k] += __ldcg(p.partials + (int64_t)(rb + q) * 3 + k);
-                    }
-                }
-                block_sum_dyn<3>(acc, s_red);
-                if (tid == 0) {
-                    const int64_t row = (int64_t)s_sp.sample_id * p.series_ld;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k)
-                        if (want[k]) p.series[row + (t + k) / p.qoi_every] = acc[k] * s_sp.u_ref_inv2;
-                    p.counters[j] = 0;
-                }
-            }
-        }
-    }
-}
-
-
-// ------------------------------------------------------------------------------------------
-// Three-step strips at a compile-time width W (a whole number of 64-column blocks): the schedule of
-// strip3_kernel with every shared-memory and global address an immediate offset from a few base
-// pointers.  The rings keep two halo columns on each side of a row (RS = W + 4 floats per plane):
-// the block's first and last pairs also write their values into the opposite halo, so the gathers of
-// the edge columns read the periodic neighbours without any index wrapping.  The lattices keep each
-// row's nine populations together (row stride 9 W, population stride W), so a row's loads and the
-// push of its three destination rows are immediate offsets from one pointer per row.
-// ------------------------------------------------------------------------------------------
-// Threads per SM the register budget of the fixed-width strips is sized for (65536 registers over
-// them).  Measured on the 625 x 256^2 ensemble (kernel GLUPS at 512 / 768 / 1024 threads): FP32 230 /
-// 221 / 216 (four blocks fit the shared memory; more registers serve them best), FX16 167 / 190 / 195,
-// BF16 185 / 201 / 212 (six blocks fit; the register budget then decides how many run).
-#ifndef UQLB_STRIP3W_THREADS_F32
-#define UQLB_STRIP3W_THREADS_F32 512
-#endif
-#ifndef UQLB_STRIP3W_THREADS_16
-#define UQLB_STRIP3W_THREADS_16 1024
-#endif
-// Register staging (D == 2) holds nine more words per thread: 16-bit storage then takes the budget of
-// 768 threads (85 registers; six blocks of 128 threads still fit), where 1024 would spill.
-template <typename S, int D>
-constexpr int strip3w_min_blocks(int np) {
-    constexpr int th = sizeof(S) == 4 ? UQLB_STRIP3W_THREADS_F32 : (D == 2 ? 768 : UQLB_STRIP3W_THREADS_16);
-    return th / np < 1 ? 1 : (th / np > 16 ? 16 : th / np);
-}
-
-// D: staging of the phase-A rows ahead of their use: 0 none, 1 the next row in shared memory
-// (cp.async), 2 the next row in registers.
-template <typename S, int W, int D>
-__global__ void __launch_bounds__(W / 2, strip3w_min_blocks<S, D>(W / 2)) strip3w_kernel(KParams p) {
-    constexpr int NP = W / 2, RS = W + 4;
-    extern __shared__ __align__(16) unsigned char s5_raw[];
-    __shared__ __align__(16) SampleDev s_sp;
-    __shared__ int s_j, s_rows, s_nact, s_flag;
-    const int tid = threadIdx.x;
-    float* ring1 = reinterpret_cast<float*>(s5_raw);  // [kRing3Planes][RS]
-    float* ring2 = ring1 + kRing3Planes * RS;
-    double* s_red = reinterpret_cast<double*>(s5_raw);
-    S* stage = reinterpret_cast<S*>(ring2 + kRing3Planes * RS);  // D == 1: [9][W], the next phase-A row
-    const int t = (int)p.step_counter[0] + p.dt;
-    const int t0 = (int)p.step_counter[1];
-    if (tid == 0) {
-        const int nact = active_samples(p, t);
-        s_nact = nact;
-        s_rows = p.row_base[nact];
-    }
-    __syncthreads();
-    const int nact = s_nact, rows = s_rows;
-    const int per = (rows + gridDim.x - 1) / gridDim.x;
-    const int r0 = blockIdx.x * per, r1 = min(rows, r0 + per);
-    const bool series = p.qoi_every > 0 && p.series != nullptr;
-    const bool sr = sizeof(S) == 2 && p.stochastic != 0;
-    const int x = 2 * tid;
-    float* const r1t = ring1 + 2 + x;  // this thread's column x in ring 1 (column c sits at 2 + c)
-    float* const r2t = ring2 + 2 + x;
-    const bool first = tid == 0, last = tid == NP - 1;
-    // push offsets of the wrapped neighbour columns: node a's x - 1 and node b's x + 2
-    const int offl = first ? W - 1 : -1, offr = last ? 2 - W : 2;
-    for (int r = r0; r < r1;) {
-        __syncthreads();
-        if (tid == 0) {
-            int lo = 0, hi = nact - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (p.row_base[mid] <= r)
-                    lo = mid;
-                else
-                    hi = mid - 1;
-            }
-            s_j = lo;
-        }
-        __syncthreads();
-        const int j = s_j;
-        if (tid < 32) reinterpret_cast<uint32_t*>(&s_sp)[tid] = __ldg(reinterpret_cast<const uint32_t*>(p.samples + j) + tid);
-        __syncthreads();
-        const int rb = p.row_base[j];
-        const int ny = s_sp.ny;
-        const int ya = r - rb, yb = min(ny, r1 - rb);
-        r = rb + yb;
-        const int n = min(3, s_sp.steps - t);
-        bool want[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) want[k] = series && k < n && ((t + k) % p.qoi_every) == 0;
-        const bool second = ((p.sel[s_sp.slot] ^ ((t - t0) / 3)) & 1) != 0;
-        const S* src = static_cast<const S*>(second ? p.arena2 : p.arena) + s_sp.f_off + x;
-        S* dst = static_cast<S*>(second ? p.arena : p.arena2) + s_sp.f_off + x;
-        const float omega = (float)s_sp.omega;
-        const PackedBGK omega2 = packed_bgk(omega);
-        const uint32_t sid = (uint32_t)s_sp.sample_id;
-        const typename Storage<S>::Q qz = quanta_of<S>(p, j);
-        double red[3] = {0.0, 0.0, 0.0};
-        auto wrap = [&](int y) {
-            y += y < 0 ? ny : 0;
-            y += y < 0 ? ny : 0;
-            y -= y >= ny ? ny : 0;
-            y -= y >= ny ? ny : 0;
-            return y;
-        };
-        // FP32 stores (16-bit storage rounds whole pairs, in push)
-        auto st1 = [&](S* d, float v, int i) { Storage<S>::store(d, v, qz, i); };
-        auto st2 = [&](S* d, f2 v, int i) { pair_store<S>(d, v, qz, i); };
-        // push of the pair's post-collision populations g (step ts, row y) into the other lattice
-        auto push = [&](int y, int ts, const f2 (&g)[9]) {
-            const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
-            if constexpr (sizeof(S) == 2) {
-                // 16-bit storage: each population's pair rounded into one word (one hash per pair and
-                // step for the stochastic bits); the x-moving populations land in two columns
-                uint32_t h = 0u;
-                if (sr)
-                    h = mix32((uint32_t)(y * 9 * W + x) * 0x9E3779B1u + (uint32_t)ts * 0x85EBCA77u +
-                              sid * 0xC2B2AE3Du);
-                auto word = [&](int i) {
-                    return sr ? pair_word_sr<S>(g[i], sr_bits(h, i), qz, i) : pair_word<S>(g[i], qz, i);
-                };
-                auto put2 = [](S* at, uint32_t w) { *reinterpret_cast<uint32_t*>(at) = w; };
-                auto put_lo = [](S* at, uint32_t w) { *reinterpret_cast<uint16_t*>(at) = (uint16_t)w; };
-                auto put_hi = [](S* at, uint32_t w) { *reinterpret_cast<uint16_t*>(at) = (uint16_t)(w >> 16); };
-                uint32_t w;
-                {  // row y: populations 0, 1, 3
-                    S* R = dst + y * (9 * W);
-                    put2(R, word(0));
-                    w = word(1);
-                    put_lo(R + W + 1, w);
-                    put_hi(R + offr + W, w);
-                    w = word(3);
-                    put_lo(R + offl + 3 * W, w);
-                    put_hi(R + 3 * W, w);
-                }
-                {  // row y + 1: populations 2, 5, 6
-                    S* R = dst + yp * (9 * W);
-                    put2(R + 2 * W, word(2));
-                    w = word(5);
-                    put_lo(R + 5 * W + 1, w);
-                    put_hi(R + offr + 5 * W, w);
-                    w = word(6);
-                    put_lo(R + offl + 6 * W, w);
-                    put_hi(R + 6 * W, w);
-                }
-                {  // row y - 1: populations 4, 7, 8
-                    S* R = dst + ym * (9 * W);
-                    put2(R + 4 * W, word(4));
-                    w = word(7);
-                    put_lo(R + offl + 7 * W, w);
-                    put_hi(R + 7 * W, w);
-                    w = word(8);
-                    put_lo(R + 8 * W + 1, w);
-                    put_hi(R + offr + 8 * W, w);
-                }
-            } else {
-                float a, b;
-                {  // row y: populations 0, 1, 3
-                    S* R = dst + y * (9 * W);
-                    st2(R, g[0], 0);
-                    upk(g[1], a, b);
-                    st1(R + W + 1, a, 1);
-                    st1(R + offr + W, b, 1);
-                    upk(g[3], a, b);
-                    st1(R + offl + 3 * W, a, 3);
-                    st1(R + 3 * W, b, 3);
-                }
-                {  // row y + 1: populations 2, 5, 6
-                    S* R = dst + yp * (9 * W);
-                    st2(R + 2 * W, g[2], 2);
-                    upk(g[5], a, b);
-                    st1(R + 5 * W + 1, a, 5);
-                    st1(R + offr + 5 * W, b, 5);
-                    upk(g[6], a, b);
-                    st1(R + offl + 6 * W, a, 6);
-                    st1(R + 6 * W, b, 6);
-                }
-                {  // row y - 1: populations 4, 7, 8
-                    S* R = dst + ym * (9 * W);
-                    st2(R + 4 * W, g[4], 4);
-                    upk(g[7], a, b);
-                    st1(R + offl + 7 * W, a, 7);
-                    st1(R + 7 * W, b, 7);
-                    upk(g[8], a, b);
-                    st1(R + 8 * W + 1, a, 8);
-                    st1(R + offr + 8 * W, b, 8);
-                }
-            }
-        };
-        auto add_usq = [&](double& acc, f2 q) {
-            float a, b;
-            upk(q, a, b);
-            acc += (double)a + (double)b;
-        };
-        // ring plane offsets of row index q: the c_y = +1 / 0 / -1 groups (3 / 2 / 1 slots)
-        auto slot_p = [](int q) { return (q % 3) * 3 * RS; };
-        auto slot_z = [](int q) { return (9 + (q & 1) * 3) * RS; };
-        // the halo copy of the block's first pair (right halo: columns 0, 1 after W - 1) and last pair
-        // (left halo: columns W - 2, W - 1 before 0)
-        const int hoff = first ? W : -W;
-        auto put_ring = [&](float* rt, int q, const f2 (&g)[9]) {
-            const int op = slot_p(q), oz = slot_z(q), om = 15 * RS;
-            auto put = [&](float* at, int off, f2 v) { *reinterpret_cast<f2*>(at + off) = v; };
-            put(rt, op, g[2]);
-            put(rt, op + RS, g[5]);
-            put(rt, op + 2 * RS, g[6]);
-            put(rt, oz, g[0]);
-            put(rt, oz + RS, g[1]);
-            put(rt, oz + 2 * RS, g[3]);
-            put(rt, om, g[4]);
-            put(rt, om + RS, g[7]);
-            put(rt, om + 2 * RS, g[8]);
-            if (first || last) {
-                float* h = rt + hoff;
-                put(h, op, g[2]);
-                put(h, op + RS, g[5]);
-                put(h, op + 2 * RS, g[6]);
-                put(h, oz, g[0]);
-                put(h, oz + RS, g[1]);
-                put(h, oz + 2 * RS, g[3]);
-                put(h, om, g[4]);
-                put(h, om + RS, g[7]);
-                put(h, om + 2 * RS, g[8]);
-            }
-        };
-        // gather of row index q (population i from row q - c_iy, column x - c_ix)
-        auto gather = [&](const float* rt, int q, f2 (&g)[9]) {
-            const float* pp = rt + slot_p(q - 1);
-            const float* pz = rt + slot_z(q);
-            const float* pm = rt + 15 * RS;
-            g[0] = *reinterpret_cast<const f2*>(pz);
-            g[1] = pk(pz[RS - 1], pz[RS]);
-            g[3] = pk(pz[2 * RS + 1], pz[2 * RS + 2]);
-            g[2] = *reinterpret_cast<const f2*>(pp);
-            g[5] = pk(pp[RS - 1], pp[RS]);
-            g[6] = pk(pp[2 * RS + 1], pp[2 * RS + 2]);
-            g[4] = *reinterpret_cast<const f2*>(pm);
-            g[7] = pk(pm[RS + 1], pm[RS + 2]);
-            g[8] = pk(pm[2 * RS - 1], pm[2 * RS]);
-        };
-        if (n == 1) {
-            for (int y = ya; y < yb; ++y) {
-                const S* s0 = src + y * (9 * W);
-                f2 g[9];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) g[i] = pair_load<S>(s0 + i * W, qz, i);
-                f2 q;
-                collide_packed(g, omega2, want[0] ? &q : nullptr);
-                if (want[0]) add_usq(red[0], q);
-                push(y, t, g);
-            }
-        } else {
-            const int a0 = ya - (n - 1);
-            auto fetch = [&](int qa) {
-                if (a0 + qa <= yb + n - 2) {
-                    const S* s0 = src + wrap(a0 + qa) * (9 * W);
-                    S* st = stage + x;
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) cp_async<2 * sizeof(S)>(st + i * W, s0 + i * W);
-                }
-                cp_async_commit();
-            };
-            (void)fetch;
-            // D == 2: the next phase-A row's pairs are loaded into registers one row ahead, so their
-            // latency overlaps the rest of the row's work and its barriers
-            using Raw = PairRaw<S>;
-            Raw pre[9];
-            auto fetch_regs = [&](int row) {
-                if (row - a0 <= yb + n - 2 - a0) {
-                    const Raw* s0 = reinterpret_cast<const Raw*>(src + wrap(row) * (9 * W));
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) pre[i] = __ldg(s0 + i * (W / 2));
-                }
-            };
-            (void)fetch_regs;
-            auto phase_a = [&](int row) {
-                const int qa = row - a0;
-                f2 g[9];
-                if constexpr (D == 1) {
-                    cp_async_wait<0>();
-                    const S* st = stage + x;
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) g[i] = pair_load<S>(st + i * W, qz, i);
-                    fetch(qa + 1);
-                } else if constexpr (D == 2) {
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) g[i] = pair_from_raw<S>(pre[i], qz, i);
-                    fetch_regs(row + 1);
-                } else {
-                    const S* s0 = src + wrap(row) * (9 * W);
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) g[i] = pair_load<S>(s0 + i * W, qz, i);
-                }
-                f2 qq;
-                const bool w = want[0] && row >= ya && row < yb;
-                collide_packed(g, omega2, w ? &qq : nullptr);
-                if (w) add_usq(red[0], qq);
-                put_ring(r1t, row - ya + 4, g);
-            };
-            if constexpr (D == 1) fetch(0);
-            if constexpr (D == 2) fetch_regs(a0);
-            if (n == 3) {
-                phase_a(ya - 2);
-                phase_a(ya - 1);
-                for (int y = ya - 2; y < yb; ++y) {
-                    phase_a(y + 2);
-                    __syncthreads();
-                    {
-                        f2 g[9];
-                        gather(r1t, y + 1 - ya + 4, g);
-                        f2 qq;
-                        const bool w = want[1] && y + 1 >= ya && y + 1 < yb;
-                        collide_packed(g, omega2, w ? &qq : nullptr);
-                        if (w) add_usq(red[1], qq);
-                        put_ring(r2t, y + 1 - ya + 4, g);
-                    }
-                    __syncthreads();
-                    if (y >= ya) {
-                        f2 g[9];
-                        gather(r2t, y - ya + 4, g);
-                        f2 qq;
-                        collide_packed(g, omega2, want[2] ? &qq : nullptr);
-                        if (want[2]) add_usq(red[2], qq);
-                        push(y, t + 2, g);
-                    }
-                }
-            } else {
-                phase_a(ya - 1);
-                for (int y = ya - 1; y < yb; ++y) {
-                    phase_a(y + 1);
-                    __syncthreads();
-                    if (y >= ya) {
-                        f2 g[9];
-                        gather(r1t, y - ya + 4, g);
-                        f2 qq;
-                        collide_packed(g, omega2, want[1] ? &qq : nullptr);
-                        if (want[1]) add_usq(red[1], qq);
-                        push(y, t + 1, g);
-                    }
-                    __syncthreads();
-                }
-            }
-            if constexpr (D == 1) cp_async_wait<0>();
-        }
-        if (want[0] || want[1] || want[2]) {
-            __syncthreads();
-            block_sum_dyn<3>(red, s_red);
-            if (tid == 0) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) p.partials[(int64_t)(rb + ya) * 3 + k] = red[k];
-                __threadfence();
-                const int prev = atomicAdd(p.counters + j, yb - ya);
-                s_flag = (prev + (yb - ya) == ny);
-            }
-            __syncthreads();
-            if (s_flag) {
-                __threadfence();
-                double acc[3] = {0.0, 0.0, 0.0};
-                for (int q = tid; q < ny; q += NP) {
-                    if (q == 0 || (rb + q) % per == 0) {
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) acc[k] += __ldcg(p.partials + (int64_t)(rb + q) * 3 + k);
-                    }
-                }
-                block_sum_dyn<3>(acc, s_red);
-                if (tid == 0) {
-                    const int64_t row = (int64_t)s_sp.sample_id * p.series_ld;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k)
-                        if (want[k]) p.series[row + (t + k) / p.qoi_every] = acc[k] * s_sp.u_ref_inv2;
-                    p.counters[j] = 0;
-                }
-            }
-        }
-    }
-}
-
+#include "strip_regs.cuh"
 
 // ------------------------------------------------------------------------------------------
 // Channel samples held on chip: one thread-block cluster per sample runs its whole time loop.
@@ -3318,11 +2599,6 @@ cudaError_t launch_bouzidi_force_s(const KParams& p, const BatchGeometry& g, cud
     return cudaGetLastError();
 }
 
-template <typename S>
-size_t strip3_smem(int nx) {
-    return (size_t)2 * kRing3Planes * nx * sizeof(float) + (size_t)Strip3Tune<S>::depth * 9 * nx * sizeof(S);
-}
-
 // Carveout (percent of the largest share) that selects configuration `kb`: rounded down, since the
 // driver rounds the share up to the next configuration.
 inline int carveout_pct(int kb) { return kb * 100 / 228; }
@@ -3336,27 +2612,6 @@ inline void strip_launch_shape(const StripBlocks& sb, const BatchGeometry& g, in
     k = std::max(k, smem_config_for((size_t)b * sb.per_block));
     *bps = b;
     *kb = k;
-}
-
-// Launch of a row-strip kernel over min(total rows, bps x SMs) blocks with the shared-memory share
-// as a launch attribute (it holds for this launch only, also inside a captured graph).
-template <typename K>
-cudaError_t launch_strip_kernel(K kernel, const StripBlocks& sb, const BatchGeometry& g, int threads, size_t smem,
-                                const KParams& p, cudaStream_t s) {
-    int bps = 0, kb = 0;
-    strip_launch_shape(sb, g, &bps, &kb);
-    const int64_t resident = (int64_t)bps * sm_count();
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(g.total_rows, resident)));
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    at[0].val.sharedMemCarveout = (unsigned)carveout_pct(kb);
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
 // Blocks per SM of a kernel with `dyn` bytes of dynamic shared memory at `threads` threads: the
@@ -3376,93 +2631,88 @@ StripBlocks strip_blocks_of(K kernel, int threads, size_t dyn, int default_kb) {
     return r;
 }
 
-// Blocks per SM of the three-step strips at width nx (once per width).
-template <typename S, bool GENERIC>
-const StripBlocks& strip3_generic_blocks(int nx) {
-    const int np = strip_threads(nx), rw = 2 * np;
-    static StripBlocks cache[1024 / 32 + 1] = {};
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(strip3_kernel<S, GENERIC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)strip3_smem<S>(Strip3Tune<S>::max_nx));
-        attr = true;
-    }
-    StripBlocks& b = cache[np / 32];
-    if (b.max_b == 0) b = strip_blocks_of(strip3_kernel<S, GENERIC>, np, strip3_smem<S>(rw), Strip3Tune<S>::carveout_kb);
+// Blocks per SM of one instantiation of the three-step strips (once).  By default the most blocks that
+// fit and the smallest shared-memory share that holds them: the rest of the 256 KB is L1, where the
+// halo columns that neighbouring windows share are found.
+template <typename S, int W, int D, bool ODD>
+const StripBlocks& strip_regs_blocks() {
+    static const StripBlocks b = strip_blocks_of(strip_regs_kernel<S, W, D, ODD>, kStripThreads, 0, -1);
     return b;
 }
 
-template <typename S, int W, int D>
-size_t strip3w_smem() {
-    return (size_t)2 * kRing3Planes * (W + 4) * sizeof(float) + (size_t)(D == 1 ? 1 : 0) * 9 * W * sizeof(S);
-}
-
-// Blocks per SM of the fixed-width three-step strips (once).
-template <typename S, int W, int D>
-const StripBlocks& strip3w_blocks() {
-    static const StripBlocks b = [] {
-        cudaFuncSetAttribute(strip3w_kernel<S, W, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)strip3w_smem<S, W, D>());
-        // register staging: by default the most blocks that fit and the smallest share that holds
-        // them (the rest of the 256 KB as L1: FP32 4 blocks and 164 KB, 0.170 against 0.202 ms per
-        // step at 228 KB)
-        return strip_blocks_of(strip3w_kernel<S, W, D>, W / 2, strip3w_smem<S, W, D>(),
-                               D == 2 ? -1 : Strip3Tune<S>::carveout_kb);
-    }();
-    return b;
-}
-
-// Staging of a fixed-width launch's phase-A rows: option 1 = none, 2 = the next row in shared memory
-// by cp.async, 3 = the next row in registers (0: the compiled default); as the kernel's D: 0, 1, 2.
-// The default is register staging (measured on the 625 x 256^2 ensemble, kernel GLUPS, none / shared
-// memory / registers: FP32 199 / 228 / 241, BF16 219 / 227 / 234, FP16 214 / 223 / 230, FX16 200 / 204
-// / 216; `def`, the runtime-width kernel's compiled staging, is not used).
-inline int strip3w_depth(int stage, int def) {
-    (void)def;
-    return stage == 1 ? 0 : (stage == 2 ? 1 : 2);
-}
-
-template <typename S, int W, int D>
-cudaError_t launch_strip3w_d(const KParams& p, const BatchGeometry& g, cudaStream_t s, bool prepare_only) {
-    const StripBlocks& sb = strip3w_blocks<S, W, D>();
+template <typename S, int W, int D, bool ODD>
+cudaError_t launch_strip_regs_d(const KParams& p, const BatchGeometry& g, cudaStream_t s, bool prepare_only,
+                                StripBlocks* blocks) {
+    const StripBlocks& sb = strip_regs_blocks<S, W, D, ODD>();
+    if (blocks != nullptr) *blocks = sb;
     if (prepare_only) return cudaGetLastError();
-    return launch_strip_kernel(strip3w_kernel<S, W, D>, sb, g, W / 2, strip3w_smem<S, W, D>(), p, s);
+    StripMap map{};
+    map.samples = g.strip_t;
+    map.warps = g.strip_g;
+    map.closed = g.strip_closed;
+    map.nx = g.strip_nx;
+    map.ny = g.strip_ny;
+    if (!map.closed) {
+        StripPacker k((g.strip_nx + 1) / 2, g.strip_t);
+        int n = 0;
+        while (k.next()) {
+            map.stretch[n++] = {(uint8_t)k.task, (uint8_t)k.lane0, (uint8_t)k.count, 0, k.first};
+            map.start[k.warp + 1] = (uint8_t)n;
+        }
+    }
+    // at most one row of a group's T samples per group of G warps
+    const int64_t rows = g.strip_ny > 0 ? (g.nsamples + g.strip_t - 1) / g.strip_t * g.strip_ny : g.total_rows;
+    const int64_t most = (rows * g.strip_g + kStripWarps - 1) / kStripWarps;
+    int bps = 0, kb = 0;
+    strip_launch_shape(sb, g, &bps, &kb);
+    const int64_t resident = std::max<int64_t>((int64_t)bps * sm_count(), (g.strip_g + kStripWarps - 1) / kStripWarps);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>(std::min(most, resident), kStripMaxWarps / kStripWarps));
+    cfg.blockDim = dim3(kStripThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[0].val.sharedMemCarveout = (unsigned)carveout_pct(kb);
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, strip_regs_kernel<S, W, D, ODD>, p, map);
 }
 
-template <typename S, int W>
-cudaError_t launch_strip3w(const KParams& p, const BatchGeometry& g, cudaStream_t s, bool prepare_only) {
-    switch (strip3w_depth(g.strip_stage, Strip3Tune<S>::depth)) {
-        case 0: return launch_strip3w_d<S, W, 0>(p, g, s, prepare_only);
-        case 1: return launch_strip3w_d<S, W, 1>(p, g, s, prepare_only);
-        default: return launch_strip3w_d<S, W, 2>(p, g, s, prepare_only);
+// Staging of a launch's phase-0 rows: option 1 = none, 2 = the next rows in shared memory by cp.async,
+// 3 = the next row in registers (0: the storage's default).  Staging options are compiled for the
+// widths with a compile-time instantiation.
+template <typename S, int W, bool ODD>
+cudaError_t launch_strip_regs_w(const KParams& p, const BatchGeometry& g, int stage, cudaStream_t s, bool prepare_only,
+                                StripBlocks* blocks) {
+    if constexpr (W == 0) {
+        return launch_strip_regs_d<S, W, kStripDefaultD<S, ODD>, ODD>(p, g, s, prepare_only, blocks);
+    } else {
+        switch (stage == 0 ? kStripDefaultD<S, ODD> + 1 : stage) {
+            case 1: return launch_strip_regs_d<S, W, 0, ODD>(p, g, s, prepare_only, blocks);
+            case 2: return launch_strip_regs_d<S, W, 1, ODD>(p, g, s, prepare_only, blocks);
+            default: return launch_strip_regs_d<S, W, 2, ODD>(p, g, s, prepare_only, blocks);
+        }
     }
 }
 
-template <typename S, int W>
-const StripBlocks& strip3w_blocks_at(int d) {
-    return d == 0 ? strip3w_blocks<S, W, 0>() : (d == 1 ? strip3w_blocks<S, W, 1>() : strip3w_blocks<S, W, 2>());
+template <typename S>
+cudaError_t launch_strip_regs(const KParams& p, const BatchGeometry& g, int stage, cudaStream_t s, bool prepare_only,
+                              StripBlocks* blocks) {
+    if (g.strip_nx < 2 || g.strip_nx > kStripMaxNx<S>) return cudaErrorInvalidConfiguration;
+    switch (strip3_fixed_width(g.strip_nx) ? g.strip_nx : 0) {
+        case 64: return launch_strip_regs_w<S, 64, false>(p, g, stage, s, prepare_only, blocks);
+        case 128: return launch_strip_regs_w<S, 128, false>(p, g, stage, s, prepare_only, blocks);
+        case 256: return launch_strip_regs_w<S, 256, false>(p, g, stage, s, prepare_only, blocks);
+        case 512: return launch_strip_regs_w<S, 512, false>(p, g, stage, s, prepare_only, blocks);
+        case 1024: return launch_strip_regs_w<S, 1024, false>(p, g, stage, s, prepare_only, blocks);
+    }
+    if (g.strip_nx & 1) return launch_strip_regs_w<S, 0, true>(p, g, stage, s, prepare_only, blocks);
+    return launch_strip_regs_w<S, 0, false>(p, g, stage, s, prepare_only, blocks);
 }
 
 template <typename S>
 cudaError_t launch_strip3_s(const KParams& p, const BatchGeometry& g, cudaStream_t s, bool prepare_only) {
-    const int np = strip_threads(g.strip_nx);
-    if (g.strip_nx < 2 || 2 * np > Strip3Tune<S>::max_nx) return cudaErrorInvalidConfiguration;
-    const bool generic = g.strip_nx != 2 * np;
-    if (strip3_fixed_width(g.strip_nx)) {
-        // the widths with a compile-time instantiation (immediate addressing)
-        switch (g.strip_nx) {
-            case 64: return launch_strip3w<S, 64>(p, g, s, prepare_only);
-            case 128: return launch_strip3w<S, 128>(p, g, s, prepare_only);
-            case 256: return launch_strip3w<S, 256>(p, g, s, prepare_only);
-            case 512: return launch_strip3w<S, 512>(p, g, s, prepare_only);
-            default: return launch_strip3w<S, 1024>(p, g, s, prepare_only);
-        }
-    }
-    const StripBlocks& sb =
-        generic ? strip3_generic_blocks<S, true>(g.strip_nx) : strip3_generic_blocks<S, false>(g.strip_nx);
-    if (prepare_only) return cudaGetLastError();
-    if (generic) return launch_strip_kernel(strip3_kernel<S, true>, sb, g, np, strip3_smem<S>(2 * np), p, s);
-    return launch_strip_kernel(strip3_kernel<S, false>, sb, g, np, strip3_smem<S>(2 * np), p, s);
+    return launch_strip_regs<S>(p, g, g.strip_stage, s, prepare_only, nullptr);
 }
 
 // Blocks per SM of the three-step strips of batch g at staging option `stage` (fixed widths only;
@@ -3472,23 +2722,8 @@ bool strip3_blocks_s(const BatchGeometry& g, int stage, StripBlocks* out) {
     if constexpr (sizeof(S) == 8) {
         return false;
     } else {
-        const int np = strip_threads(g.strip_nx);
-        if (!g.strips || g.spl != 3 || g.strip_nx < 2 || 2 * np > Strip3Tune<S>::max_nx) return false;
-        if (strip3_fixed_width(g.strip_nx)) {
-            const int d = strip3w_depth(stage, Strip3Tune<S>::depth);
-            switch (g.strip_nx) {
-                case 64: *out = strip3w_blocks_at<S, 64>(d); break;
-                case 128: *out = strip3w_blocks_at<S, 128>(d); break;
-                case 256: *out = strip3w_blocks_at<S, 256>(d); break;
-                case 512: *out = strip3w_blocks_at<S, 512>(d); break;
-                default: *out = strip3w_blocks_at<S, 1024>(d); break;
-            }
-            return true;
-        }
-        if (stage != 0) return false;
-        *out = g.strip_nx != 2 * np ? strip3_generic_blocks<S, true>(g.strip_nx)
-                                     : strip3_generic_blocks<S, false>(g.strip_nx);
-        return true;
+        if (!g.strips || g.spl < 3 || (stage != 0 && !strip3_fixed_width(g.strip_nx))) return false;
+        return launch_strip_regs<S>(KParams{}, g, stage, nullptr, true, out) == cudaSuccess;
     }
 }
 
@@ -3496,7 +2731,7 @@ template <typename S>
 cudaError_t launch_two_step_s(const KParams& p, const BatchGeometry& g, cudaStream_t s, bool prepare_only) {
     if (g.strips) {
         if constexpr (sizeof(S) == 8) return cudaErrorInvalidConfiguration;
-        else if (g.spl == 3) return launch_strip3_s<S>(p, g, s, prepare_only);
+        else if (g.spl >= 3) return launch_strip3_s<S>(p, g, s, prepare_only);
         else return launch_strip_s<S>(p, g, s, prepare_only);
     }
     return launch_step2_s<S>(p, g, s, prepare_only);

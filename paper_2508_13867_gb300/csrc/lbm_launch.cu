@@ -48,6 +48,7 @@ KParams make_params(const BatchBuffers& b, const BatchGeometry& g, const RunOutp
     p.arena2 = b.arena2;
     p.sel = b.sel;
     p.row_base = b.row_base;
+    p.kpart = b.kpart;
     p.samples = b.samples;
     p.init = b.init;
     p.steps_sorted = b.steps_sorted;
@@ -99,7 +100,7 @@ bool strip_supported(int storage, int nx) {
 bool strip3_supported(int storage, int nx) {
     if (storage == UQLB_F64 || nx < 2) return false;
     const int rw = 2 * strip_threads(nx);
-    return rw <= (storage == UQLB_F32 ? Strip3Tune<float>::max_nx : Strip3Tune<__half>::max_nx);
+    return rw <= (storage == UQLB_F32 ? kStripMaxNx<float> : kStripMaxNx<__half>);
 }
 
 bool cluster_fits(int storage, int nx, int ny) {

@@ -410,7 +410,7 @@ struct BatchPlan {
     std::vector<uint32_t> masks;
     size_t off_arena = 0, off_arena2 = 0, off_sel = 0, off_rowbase = 0, off_bcpop = 0, off_samples = 0, off_init = 0, off_steps = 0, off_masks = 0, off_side = 0,
            off_partials = 0, off_counters = 0, off_done = 0, off_steps_run = 0, off_cd_prev = 0,
-           off_step_counter = 0, off_flag = 0, off_streak = 0, off_sync = 0, total = 0;
+           off_step_counter = 0, off_flag = 0, off_streak = 0, off_sync = 0, off_kpart = 0, total = 0;
     BatchGeometry geom{};
     int n_steady = 0;
     bool uniform_size = true;
@@ -447,6 +447,32 @@ int validate_sample(const uqlb_sample& s, int64_t idx, std::string& why) {
     }
     why = buf;
     return UQLB_ERR_ARG;
+}
+
+// Three-step strips: samples T side by side over G warps.  A row of an even number of columns that fits a
+// warp closes on itself (32 / U samples per warp); others take the T of 1..6 (at most n, at most 64
+// warps) with the largest share of useful lanes, T U / 32 G, the smallest on ties.
+void strip_lanes(int nx, int64_t n, int* T, int* G, int* closed) {
+    const int U = (nx + 1) / 2;
+    *T = *G = 1;
+    *closed = 0;
+    if (nx % 2 == 0 && U <= 32) {
+        *closed = 1;
+        *T = (int)std::min<int64_t>(32 / U, n);
+        return;
+    }
+    double best = 0.0;
+    for (int t = 1; t <= kStripGroupSamples && t <= n; ++t) {
+        StripPacker k(U, t);
+        while (k.next()) {
+        }
+        const int g = k.warp + 1;
+        const double share = (double)t * U / (32.0 * g);
+        if (g > kStripGroupWarps || share < best + 1e-9) continue;
+        best = share;
+        *T = t;
+        *G = g;
+    }
 }
 
 // ids: the caller's index of each sample (the output row), nullptr for 0..n-1.
@@ -513,7 +539,7 @@ int plan_batch(const uqlb_sample* smp, int64_t n, const uqlb_run_opts* o, BatchP
     const int spl = !two ? 1
                          : ((strip3_ok && (scheme == UQLB_SCHEME_THREE_STEP_STRIPS ||
                                            (scheme == UQLB_SCHEME_AUTO && kAutoThreeStep)))
-                                ? 3
+                                ? strip3_steps(storage)
                                 : 2);
     auto supported = [&](int r, int q) {
         return two ? geometry_supported2(storage, r, q) : geometry_supported(storage, mixed, r, q);
@@ -706,6 +732,19 @@ int plan_batch(const uqlb_sample* smp, int64_t n, const uqlb_run_opts* o, BatchP
     P.off_flag = take(sizeof(int32_t));
     P.off_streak = take(sizeof(int32_t) * n);
     P.off_sync = take(64);  // barrier count, generation, error word, ticket counter
+    // three-step strips: how rows are laid over warps, and the partial sums of K (behind everything a
+    // resumed run needs, so that a saved workspace keeps its layout)
+    int strip_t = 1, strip_g = 1, strip_closed = 0;
+    bool uniform_ny = true;
+    for (int64_t k = 1; k < n; ++k) uniform_ny = uniform_ny && smp[k].ny == smp[0].ny;
+    if (strips) {  // sized alike for the two-step strips, which a run may change to when it is resumed
+        strip_lanes(smp[0].nx, uniform_ny ? n : 1, &strip_t, &strip_g, &strip_closed);
+        // one slot per (group of samples + range, warp, sample of the group): a piece is one range's part
+        // of one group, and both grow along the pieces
+        const int64_t groups = (n + strip_t - 1) / strip_t;
+        const int64_t warps = std::min<int64_t>(total_rows * strip_g, kStripMaxWarps);
+        P.off_kpart = take((size_t)(groups * strip_g + warps) * strip_t * strip3_steps(storage) * sizeof(double));
+    }
     P.total = off;
 
     BatchGeometry& g = P.geom;
@@ -728,6 +767,10 @@ int plan_batch(const uqlb_sample* smp, int64_t n, const uqlb_run_opts* o, BatchP
     g.strips = strips ? 1 : 0;
     g.strip_nx = strips ? smp[0].nx : 0;
     g.spl = spl;
+    g.strip_t = strip_t;
+    g.strip_g = strip_g;
+    g.strip_closed = strip_closed;
+    g.strip_ny = strips && uniform_ny ? smp[0].ny : 0;
     g.cluster = cluster ? 1 : 0;
     g.cluster_nx = g.cluster_ny = 0;
     g.pad_ = 0;
@@ -741,7 +784,7 @@ int plan_batch(const uqlb_sample* smp, int64_t n, const uqlb_run_opts* o, BatchP
                   "configuration (8, 16, 32, 64, 100, 132, 164, 196, 228)";
             return UQLB_ERR_ARG;
         }
-        const bool s3 = strips && spl == 3;
+        const bool s3 = strips && spl >= 3;
         if (s3 && ss != 0 && !strip3_fixed_width(smp[0].nx)) {
             why = "strip_stage applies to the three-step strips at widths 64, 128, 256, 512 and 1024 only";
             return UQLB_ERR_ARG;
@@ -780,6 +823,7 @@ BatchBuffers carve(const BatchPlan& P, void* ws) {
     B.side_d = reinterpret_cast<double*>(b + P.off_side);
     B.bcpop = reinterpret_cast<double*>(b + P.off_bcpop);
     B.partials = reinterpret_cast<double*>(b + P.off_partials);
+    B.kpart = P.off_kpart ? reinterpret_cast<double*>(b + P.off_kpart) : nullptr;
     B.counters = reinterpret_cast<int32_t*>(b + P.off_counters);
     B.done = reinterpret_cast<int32_t*>(b + P.off_done);
     B.steps_run = reinterpret_cast<int32_t*>(b + P.off_steps_run);
@@ -1563,7 +1607,7 @@ int uqlb_autotune(uqlb_ctx* ctx, const uqlb_sample* samples, int64_t n, const uq
         const bool two = g0.two_step != 0;
         spl = two ? std::max(g0.spl, 2) : 1;
         const int scheme = !two ? UQLB_SCHEME_ONE_STEP
-                                : (g0.strips ? (g0.spl == 3 ? UQLB_SCHEME_THREE_STEP_STRIPS : UQLB_SCHEME_TWO_STEP_STRIPS)
+                                : (g0.strips ? (g0.spl >= 3 ? UQLB_SCHEME_THREE_STEP_STRIPS : UQLB_SCHEME_TWO_STEP_STRIPS)
                                              : UQLB_SCHEME_TWO_STEP_TILES);
         if (scheme == UQLB_SCHEME_THREE_STEP_STRIPS) {
             // staging option x blocks per SM (the most that fit and up to three fewer) x share (the
@@ -1751,7 +1795,7 @@ int uqlb_run_batch(uqlb_ctx* ctx, const uqlb_sample* samples, int64_t n, const u
     ctx->last_scheme = !groups.empty() ? UQLB_SCHEME_GROUPED
                        : P0.geom.cluster ? UQLB_SCHEME_CLUSTER
                        : !P0.geom.two_step ? UQLB_SCHEME_ONE_STEP
-                       : (P0.geom.strips ? (P0.geom.spl == 3 ? UQLB_SCHEME_THREE_STEP_STRIPS : UQLB_SCHEME_TWO_STEP_STRIPS)
+                       : (P0.geom.strips ? (P0.geom.spl >= 3 ? UQLB_SCHEME_THREE_STEP_STRIPS : UQLB_SCHEME_TWO_STEP_STRIPS)
                                          : UQLB_SCHEME_TWO_STEP_TILES);
     if (fields_dev) {
         if (!uniform_size) return set_err(ctx, UQLB_ERR_ARG, "run_batch: field output needs one lattice size");

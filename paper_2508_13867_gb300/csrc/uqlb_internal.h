@@ -74,6 +74,7 @@ struct BatchBuffers {
     double* side_d;          // outlet velocities (double pairs, FP64 storage)
     double* bcpop;           // interpolated inlet/outlet: next state of the end columns, 9 per node
     double* partials;        // [tiles x 3] per-tile QoI partial sums
+    double* kpart;           // three-step strips: partial sums of K per (range, warp, sample)
     int32_t* counters;       // [S] tiles finished in the current reduction
     int32_t* done;           // [S] 1 once a sample has stopped (steady state)
     int32_t* steps_run;      // [S]
@@ -104,12 +105,15 @@ struct BatchGeometry {
     int32_t any_inout;       // some sample uses the interpolated inlet/outlet
     int32_t strips;          // two-step scheme on row strips (strip2_kernel) instead of tiles
     int32_t strip_nx;        // width of every sample when strips is set
-    int32_t spl;             // time steps per launch: 1 (one-step), 2 (tiles, two-step strips), 3 (three-step strips)
+    int32_t spl;             // time steps per launch: 1 (one-step), 2 (tiles, two-step strips), 3 or 4 (three-step strips)
     int32_t cluster;         // UQLB_SCHEME_CLUSTER: one thread-block cluster per sample holds it on chip
     int32_t cluster_nx, cluster_ny;  // cluster runs: largest sample width and height
     int32_t strip_bps;       // three-step strips: resident blocks per SM (0: default)
-    int32_t strip_stage;     // three-step strips at fixed widths: 1 = no staged row, 2 = one (0: default)
+    int32_t strip_stage;     // three-step strips at fixed widths: 1 = rows not staged, 2 = shared memory, 3 = registers (0: default)
     int32_t strip_smem_kb;   // three-step strips: shared-memory share per SM in KB (0: default)
+    int32_t strip_t, strip_g;  // three-step strips: samples side by side and warps per group (StripPacker)
+    int32_t strip_closed;    // three-step strips: whole rows fit a warp, lanes wrap around
+    int32_t strip_ny;        // three-step strips: the samples' common height (0: heights differ)
     int32_t pad_;            // keeps the struct free of padding bytes (it keys the graph cache)
 };
 
@@ -180,6 +184,56 @@ inline int smem_config_for(size_t bytes) {
 inline bool strip3_fixed_width(int nx) {
     return UQLB_STRIP3_FIXED_WIDTHS && (nx == 64 || nx == 128 || nx == 256 || nx == 512 || nx == 1024);
 }
+// Time steps per launch of the three-step strips: four with FP32 storage, whose rows pass between
+// launches unrounded (18 B of HBM traffic per update; three: 24 B); 16-bit storage rounds once per
+// launch, and keeps three.
+constexpr int kStripStepsF32 = 4;
+inline int strip3_steps(int storage) { return storage == UQLB_F32 ? kStripStepsF32 : 3; }
+// Lanes of the three-step strips (strip_regs.cuh): rows of U column pairs of T samples laid end to end
+// over warps of 32 lanes, every stretch of a row with kStripHalo halo lanes on each side.  next() gives
+// the stretches in order: pairs first .. first + count - 1 of sample `task`, from lane `lane0` of `warp`.
+constexpr int kStripHalo = 2;
+constexpr int kStripMaxWarps = 4096;   // warps per launch
+struct StripPacker {
+    int U, T;
+    int warp = 0, lane0 = 0, task = 0, first = 0, count = 0;
+    int w = 0, free_ = 32, c = 0, done = 0;
+    __host__ __device__ StripPacker(int u, int t) : U(u), T(t) {}
+    __host__ __device__ bool next() {
+        if (c >= T) return false;
+        if (free_ < 2 * kStripHalo + 1) {
+            ++w;
+            free_ = 32;
+        }
+        const int room = free_ - 2 * kStripHalo, rest = U - done;
+        count = room < rest ? room : rest;
+        warp = w;
+        lane0 = 32 - free_;
+        task = c;
+        first = done;
+        free_ -= count + 2 * kStripHalo;
+        done += count;
+        if (done == U) {
+            ++c;
+            done = 0;
+        }
+        return true;
+    }
+};
+// How a launch of the three-step strips lays rows over lanes: `samples` side by side over `warps` (the
+// stretches of warp w are start[w] .. start[w + 1] - 1), or whole rows closed on themselves.
+struct StripStretch {
+    uint8_t task, lane0;
+    uint8_t count, pad_;
+    int32_t first;
+};
+constexpr int kStripGroupWarps = 64;    // most warps per group
+constexpr int kStripGroupSamples = 6;   // most samples side by side (rows that do not close)
+struct StripMap {
+    int32_t samples, warps, closed, nx, ny;  // ny: common height (0: heights differ)
+    uint8_t start[kStripGroupWarps + 4];
+    StripStretch stretch[kStripGroupWarps + kStripGroupSamples];
+};
 // Three-step strips of batch g at staging option `stage` (1: none, 2: one row, 0: default): the
 // most resident blocks per SM, the default, the default shared-memory share (KB) and the shared
 // memory per block (bytes).  False when g does not run on the three-step strips or the staging

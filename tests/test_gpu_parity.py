@@ -1204,3 +1204,34 @@ def test_cluster_scheme_steady_stop_and_resume(ens):
     res = ens.run_batch([sample_struct(s) for s in specs], storage="f32", fields=False, start_step=37, scheme="cluster")
     torch.cuda.synchronize()
     assert np.array_equal(res["qoi"].cpu().numpy(), whole["qoi"])
+
+
+@pytest.mark.parametrize("storage", ["f32", "fx16", "bf16"])
+@pytest.mark.parametrize("nx,ny,n", [(2, 2, 3), (3, 5, 7), (5, 2, 2), (31, 4, 6), (33, 3, 5), (48, 7, 4), (56, 9, 1),
+                                     (57, 6, 3), (62, 5, 33), (64, 3, 2), (66, 8, 9), (113, 5, 7), (300, 4, 5),
+                                     (1023, 3, 3)])
+def test_register_strips_over_widths_and_groups(ens, storage, nx, ny, n):
+    """Rows of every kind the three-step strips lay over warps: closed rows, rows of odd width (whose
+    pairs straddle the seam), windows of one sample and of several side by side, a last group that is
+    not full, samples that end at different steps of a launch.  FP32 fields equal the two-step strips'
+    bit for bit (same collisions, unrounded rows) and the K series to FP64 round-off of the sums.  16-bit
+    storage against the FP32 fields: a store moves a population by at most one step of its format, and the
+    moves of the at most six roundings of a run add up to at most six such steps of each of the nine
+    populations, in u and v (nine times the largest step, over rho near 1)."""
+    specs = [replace(W.tgv(nx, 13 + (k * 5) % 6, nu=0.05 + 0.01 * (k % 3), u0=0.005), ny=ny) for k in range(n)]
+    f32 = _run(ens, specs, "f32", qoi_every=3, series=True, scheme="two_step_strips")
+    if storage == "f32":
+        got = _run(ens, specs, "f32", qoi_every=3, series=True, scheme="three_step_strips")
+        assert np.array_equal(got["fields"][:, :-1], f32["fields"][:, :-1])
+        assert np.allclose(got["series"], f32["series"], rtol=1e-12, atol=0, equal_nan=True)
+        return
+    got = _run(ens, specs, storage, scheme="three_step_strips")
+    if storage == "fx16":
+        step = max(float(U.uqlb_fx16_quanta(sample_struct(s)).max()) for s in specs)
+    else:  # BF16 keeps 8 bits of a population; none exceeds w (1.5 u + ...) of the start, here 0.01
+        step = 0.01 * 2.0 ** -8
+    ok = got["qoi"][:, U.UQLB_QOI_STATUS] == 0
+    if nx == ny or storage == "bf16":
+        assert ok.all()
+    diff = np.abs(got["fields"][ok, :-1] - f32["fields"][ok, :-1])
+    assert diff.size == 0 or diff.max() < 6 * 9 * step
