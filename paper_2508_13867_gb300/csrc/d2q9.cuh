@@ -218,6 +218,55 @@ __device__ __forceinline__ void bgk(C g[9], C omega, C drho, C jx, C jy, C ux, C
     }
 }
 
+// ---- FP64 collision ---------------------------------------------------------------------------
+// GB300 issues one FP64 instruction per warp and quarter SM in 76 cycles, so FP64 lattices are bound by
+// their count of FP64 instructions alone.  The collision of moments() and bgk() with omega folded into
+// the coefficients (as PackedBGK below), 54 instead of 108 of them:
+//   1/rho by the hardware's reciprocal seed (20 bits) and one Halley step r (1 + e + e^2), e = 1 - rho r,
+//     whose error e^3 is below 2^-59 (3 FMA; the IEEE division took about 10);
+//   with h = omega/2 / rho, q = h j:  a = jx qx, s = a + jy qy (= omega w_1 4.5 j.u),
+//   X = omega w_1 drho - s/3  and per pair of opposite directions the even part
+//   E_1 = X + a, E_2 = X + s - a, E_5,6 = (omega w_1 drho + 2/3 s)/4 +- jx qy/2  (w_5 = w_1/4),
+//   g_i* = (1 - omega) g_i + (E +- omega L_i c_i.j),  g_0* = (1 - omega) g_0 + 4 X.
+// No product with a zero component of c_i is formed (0 x is not x to a compiler that keeps NaN).
+// Measured: 64 cylinder samples of 440 x 82 0.358 against 0.579 ms per step (the rest: the boundary nodes'
+// FP64 work), 5 samples of 64 x 64 6.5 against 8.6 us per step.  Against 80-bit arithmetic over 400 to 600
+// steps at u0 0.01 to 0.05 the velocity's error is 0.45 to 1.0 times that of the two functions above.
+struct Bgk64 {
+    double omc, ow1, h, l1, l5;
+};
+__device__ __forceinline__ double rcp64(double v) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+    const double e = fma(-v, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+// rinv: 1/rho (u = j rinv where a caller needs it).
+__device__ __forceinline__ void collide64(double (&g)[9], const Bgk64& k, double& jx, double& jy, double& rinv) {
+    const double drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
+    const double d57 = g[5] - g[7], d68 = g[6] - g[8];
+    jx = (g[1] - g[3]) + (d57 - d68);
+    jy = (g[2] - g[4]) + (d57 + d68);
+    rinv = rcp64(1.0 + drho);
+    const double h = k.h * rinv;
+    const double qx = h * jx, qy = h * jy;
+    const double a = jx * qx, s = fma(jy, qy, a);
+    const double od = k.ow1 * drho;
+    const double X = fma(s, -1.0 / 3.0, od);
+    const double Y = 0.25 * fma(s, 2.0 / 3.0, od), c = jx * qy;
+    const double E1 = X + a, E2 = fma(jy, qy, X), E5 = fma(c, 0.5, Y), E6 = fma(c, -0.5, Y);
+    const double j5 = jx + jy, j6 = jy - jx;
+    g[0] = fma(g[0], k.omc, 4.0 * X);
+    g[1] = fma(g[1], k.omc, fma(k.l1, jx, E1));
+    g[3] = fma(g[3], k.omc, fma(-k.l1, jx, E1));
+    g[2] = fma(g[2], k.omc, fma(k.l1, jy, E2));
+    g[4] = fma(g[4], k.omc, fma(-k.l1, jy, E2));
+    g[5] = fma(g[5], k.omc, fma(k.l5, j5, E5));
+    g[7] = fma(g[7], k.omc, fma(-k.l5, j5, E5));
+    g[6] = fma(g[6], k.omc, fma(k.l5, j6, E6));
+    g[8] = fma(g[8], k.omc, fma(-k.l5, j6, E6));
+}
+
 // ---- Two nodes at once in packed FP32 (sm_100+ f32x2 arithmetic) ---------------------------
 // A 64-bit register holds one value of node a (low half) and of node b (high half); each packed
 // add / sub / mul / fma rounds both halves as the scalar instruction does.

@@ -104,6 +104,20 @@ __device__ __forceinline__ C inflow(const SampleDev& sp, C yy, int t) {
     return C(4) * C(sp.uin_max) * ramp * yy * (H - yy) / (H * H);
 }
 
+// The same in FP64 split for the three directions of an inlet node: the factor of the profile, once per
+// node and step (its cosine and divisions are some fifty FP64 instructions, on the warps that every
+// step waits for), and the profile at y + (1 - cy)/2.
+__device__ __forceinline__ double inflow_factor(const SampleDev& sp, int t) {
+    double ramp = 1.0;
+    if (sp.ramp_steps > 0.0 && (double)t < sp.ramp_steps) ramp = 0.5 * (1.0 - cospi((double)t / sp.ramp_steps));
+    const double H = (double)sp.ny;
+    return sp.uin_max * ramp / (H * H);
+}
+__device__ __forceinline__ double inflow_at(const SampleDev& sp, double factor, int y, int cyi) {
+    const int a = 2 * y + 1 - cyi;  // twice the height
+    return factor * ((double)a * (double)(2 * sp.ny - a));
+}
+
 // ---- Bouzidi linear interpolated bounce-back on the obstacle (Sec. 8.1 cylinder surface) ----
 // A link from fluid node x along c_i into the obstacle meets the circle at the fraction q of its
 // length; the population returning to x is 2q g*_i(x) + (1 - 2q) g_i(x, t+1) for q < 1/2 and
@@ -161,11 +175,12 @@ __device__ __forceinline__ C bouzidi_local(const InitDev& in, int x, int y, int 
 
 // Shifted incoming population of direction i at node (x, y) for the stream (tp -> tp + 1),
 // given the slot layout left by an even step at time tp: g_i*(z) sits at (z, slot opp(i)).
-// ub: velocity of the outlet node at time tp.
+// ub: velocity of the outlet node at time tp; in_factor: FP64 storage, inflow_factor of an inlet node.
 template <typename S>
 __device__ __forceinline__ typename Storage<S>::C read_incoming(
     const S* base, const SampleDev& sp, const uint32_t* mask, int x, int y, int i, int tp,
-    typename Storage<S>::C ubx, typename Storage<S>::C uby, bool chan, const typename Storage<S>::Q& qz) {
+    typename Storage<S>::C ubx, typename Storage<S>::C uby, bool chan, const typename Storage<S>::Q& qz,
+    double in_factor) {
     using C = typename Storage<S>::C;
     const int64_t plane = sp.plane;
     const int pitch = sp.pitch;
@@ -181,6 +196,7 @@ __device__ __forceinline__ typename Storage<S>::C read_incoming(
         const C mine = Storage<S>::load(base + i * plane + own, qz, i);  // g_opp(i)*(x, tp)
         if (cls == kWall || cls == kSolid) return mine;
         if (cls == kInlet) {
+            if constexpr (sizeof(C) == 8) return mine + C(6) * wgt<C>(i) * C(cx(i)) * inflow_at(sp, in_factor, y, cy(i));
             const C yy = C(y) + C(0.5) - C(0.5) * C(cy(i));
             return mine + C(6) * wgt<C>(i) * C(cx(i)) * inflow<C>(sp, yy, tp);
         }
@@ -387,8 +403,11 @@ __device__ __forceinline__ void node_load(const KParams& p, const SampleDev& sp,
             }
         }
         g[0] = Storage<S>::load(base + (nb.row[1] + x), qz, 0);
+        double in_factor = 0.0;
+        if (sizeof(C) == 8 && x == 0) in_factor = inflow_factor(sp, t - 1);
 #pragma unroll
-        for (int i = 1; i < 9; ++i) g[i] = read_incoming<S>(base, sp, mask, x, y, i, t - 1, ubx, uby, chan, qz);
+        for (int i = 1; i < 9; ++i)
+            g[i] = read_incoming<S>(base, sp, mask, x, y, i, t - 1, ubx, uby, chan, qz, in_factor);
         if (links) bouzidi_complete(*bz, x, y, links, g);
     }
 }
@@ -399,7 +418,7 @@ __device__ __forceinline__ void node_update(const KParams& p, const SampleDev& s
                                             int x, int y, int t, bool chan, bool want_k, bool want_f,
                                             const Nbr& nb, const InitDev* bz, uint32_t links,
                                             typename Storage<S>::C (&g)[9], double (&red)[3],
-                                            const typename Storage<S>::Q& qz) {
+                                            const typename Storage<S>::Q& qz, const Bgk64& k64) {
     using C = typename Storage<S>::C;
     const int own = nb.row[1] + x;
     const int plane = (int)sp.plane;
@@ -415,8 +434,19 @@ __device__ __forceinline__ void node_update(const KParams& p, const SampleDev& s
         else
             Storage<S>::store(ptr, v, qz, i);
     };
-    C drho, jx, jy, ux, uy;
-    moments(g, drho, jx, jy, ux, uy);
+    C ux, uy;
+    if constexpr (sizeof(C) == 8) {
+        C jx, jy, rinv;
+        collide64(g, k64, jx, jy, rinv);
+        if (want_k || (chan && x == sp.nx - 1)) {
+            ux = jx * rinv;
+            uy = jy * rinv;
+        }
+    } else {
+        C drho, jx, jy;
+        moments(g, drho, jx, jy, ux, uy);
+        bgk(g, (C)sp.omega, drho, jx, jy, ux, uy);
+    }
     if (want_k) red[0] += (double)(ux * ux + uy * uy);
     if (chan && !ODD && x == sp.nx - 1) {
         if (sizeof(C) == 8) {
@@ -427,7 +457,6 @@ __device__ __forceinline__ void node_update(const KParams& p, const SampleDev& s
             p.side[2 * (sp.side_off + y) + 1] = (float)uy;
         }
     }
-    bgk(g, (C)sp.omega, drho, jx, jy, ux, uy);
     if (want_f && mask != nullptr) {
         C fx = C(0), fy = C(0);
 #pragma unroll
@@ -466,6 +495,8 @@ __device__ __forceinline__ void node_update(const KParams& p, const SampleDev& s
         return;
     }
     put(base + own, g[0], 0);
+    double in_factor = 0.0;
+    if (sizeof(C) == 8 && x == 0) in_factor = inflow_factor(sp, t);
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
         int dx = x + cx(i), dy = y + cy(i);
@@ -480,8 +511,12 @@ __device__ __forceinline__ void node_update(const KParams& p, const SampleDev& s
             } else if (cls == kWall || cls == kSolid) {
                 put(base + o * plane + own, g[i], i);
             } else if (cls == kInlet) {
-                const C yy = C(y) + C(0.5) - C(0.5) * C(cy(o));
-                put(base + o * plane + own, g[i] + C(6) * wgt<C>(o) * C(cx(o)) * inflow<C>(sp, yy, t), i);
+                C uw;
+                if constexpr (sizeof(C) == 8)
+                    uw = inflow_at(sp, in_factor, y, cy(o));
+                else
+                    uw = inflow<C>(sp, C(y) + C(0.5) - C(0.5) * C(cy(o)), t);
+                put(base + o * plane + own, g[i] + C(6) * wgt<C>(o) * C(cx(o)) * uw, i);
             } else {
                 const C cu = C(cx(o)) * ux + C(cy(o)) * uy;
                 put(base + o * plane + own, -g[i] + wgt<C>(o) * (C(9) * cu * cu - C(3) * (ux * ux + uy * uy)), i);
@@ -569,6 +604,11 @@ __device__ __forceinline__ void process_tile(const KParams& p, int t, int tile, 
     }
     const uint32_t* mask = (!inner_tile && sp.mask_off >= 0) ? p.masks + sp.mask_off : nullptr;
     S* base = static_cast<S*>(p.arena) + sp.f_off;
+    Bgk64 k64{};
+    if constexpr (sizeof(C) == 8) {
+        const InitDev& in = p.init[j];
+        k64 = {__ldg(&in.bgk_omc), __ldg(&in.bgk[0]), __ldg(&in.bgk[1]), __ldg(&in.bgk[2]), __ldg(&in.bgk_l5)};
+    }
 
     const InitDev* bz = (!inner_tile && sp.bouzidi && mask != nullptr) ? p.init + j : nullptr;
     C g[NPT][9];
@@ -601,7 +641,7 @@ __device__ __forceinline__ void process_tile(const KParams& p, int t, int tile, 
     for (int k = 0; k < NPT; ++k)
         if (act[k])
             node_update<S, ODD>(p, sp, base, mk[k], x0 + kTileCols * k, y, t, nc[k], want_k, want_f, nb[k], bz, lk[k],
-                                g[k], red, qz);
+                                g[k], red, qz, k64);
 
     if (want_k || want_f) {
         double tot[3];
@@ -2109,7 +2149,8 @@ __global__ void __launch_bounds__(256) finalize_kernel(KParams p, int64_t total_
                     g[0] = Storage<S>::load(base + own, qz, 0);
 #pragma unroll
                     for (int i = 1; i < 9; ++i)
-                        g[i] = read_incoming<S>(base, sp, mask, x, y, i, T - 1, ubx, uby, chan, qz);
+                        g[i] = read_incoming<S>(base, sp, mask, x, y, i, T - 1, ubx, uby, chan, qz,
+                                                sizeof(C) == 8 && chan && x == 0 ? inflow_factor(sp, T - 1) : 0.0);
                 }
                 const uint32_t links = bz != nullptr ? obstacle_links(sp, *bz, mask, x, y) : 0u;
                 if (links && T > 0) bouzidi_complete(*bz, x, y, links, g);
@@ -2245,7 +2286,8 @@ __global__ void __launch_bounds__(256) bouzidi_force_kernel(KParams p) {
                 const C q = link_q<C>(in, x, y, i);
                 if (q < C(0.5)) {
                     const C gi = prev_odd ? Storage<S>::load(base + i * sp.plane + own, qz, i)
-                                          : read_incoming<S>(base, sp, mask, x, y, i, s - 1, ubx, uby, true, qz);
+                                          : read_incoming<S>(base, sp, mask, x, y, i, s - 1, ubx, uby, true, qz,
+                                                             sizeof(C) == 8 && x == 0 ? inflow_factor(sp, s - 1) : 0.0);
                     back += (C(1) - C(2) * q) * gi;
                 }
                 const C parked = Storage<S>::load(base + i * sp.plane + (int64_t)(y + cy(i)) * sp.pitch + (x + cx(i)), qz, i);

@@ -688,6 +688,17 @@ int plan_batch(const uqlb_sample* smp, int64_t n, const uqlb_run_opts* o, BatchP
                 P.init[j].inv_quanta[c] = (float)(1.0 / q[c]);
             }
         }
+        if (storage == UQLB_F64) {
+            // relaxation constants of collide64(): omega folded into the equilibrium's coefficients, the
+            // diagonals' odd one such that 2 omega L_1 + 4 omega L_5 = omega exactly
+            InitDev& in = P.init[j];
+            in.bgk_omc = 1.0 - d.omega;
+            in.bgk[0] = d.omega / 9.0;
+            in.bgk[1] = 0.5 * d.omega;
+            in.bgk[2] = d.omega / 3.0;
+            in.bgk[3] = 0.0;
+            in.bgk_l5 = 0.25 * (d.omega - 2.0 * in.bgk[2]);
+        }
         P.init[j].u0 = s.u0;
         P.init[j].amp2 = s.amp2;
         P.init[j].amp3 = s.amp3;

@@ -50,14 +50,20 @@ __host__ __device__ inline int mask_words(const SampleDev& s) { return (s.nx + 3
 // Bouzidi links, which are rare: only nodes inside bbox look at it).
 struct alignas(16) InitDev {
     double u0, amp2, amp3;
-    double pad;
+    double bgk_omc;  // FP64 storage: 1 - omega (collide64)
     double pert[4];  // perturbed TGV amplitudes zeta_00, zeta_01, zeta_10, zeta_11
     double cyl_cx, cyl_cy, cyl_r;
-    double pad2;
+    double bgk_l5;   // FP64 storage: the diagonals' odd coefficient
     int32_t bbox[4];  // x0, x1, y0, y1 (inclusive): the only nodes that can have obstacle links
-    // 16-bit fixed-point storage: quantum of the rest, axis and diagonal populations and its inverse
-    float quanta[4];
-    float inv_quanta[4];
+    union {
+        // 16-bit fixed-point storage: quantum of the rest, axis and diagonal populations and its inverse
+        struct {
+            float quanta[4];
+            float inv_quanta[4];
+        };
+        // FP64 storage: omega / 9, omega / 2, omega / 3
+        double bgk[4];
+    };
 };
 
 // Device pointers carved out of the caller's workspace for one batch run.

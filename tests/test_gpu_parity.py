@@ -1235,3 +1235,24 @@ def test_register_strips_over_widths_and_groups(ens, storage, nx, ny, n):
         assert ok.all()
     diff = np.abs(got["fields"][ok, :-1] - f32["fields"][ok, :-1])
     assert diff.size == 0 or diff.max() < 6 * 9 * step
+
+
+@pytest.mark.parametrize("kind", ["tgv", "ramp0", "ramp1", "ramp37", "bouzidi", "interpolated"])
+def test_fp64_collision_in_fast_flows(ens, kind):
+    """FP64 storage away from the small velocities of the workloads (Mach 0.17, densities 0.1 off): the
+    folded collision, its reciprocal and the inlet's profile against the oracle.  Each of the 61 steps rounds
+    a population some 40 times by at most 2^-53 of a value of its own size, and the relaxation damps what
+    earlier steps left: 61 x 40 x 1.1e-16 = 2.7e-13, with a factor 4 for the velocity's size to the
+    populations'."""
+    if kind == "tgv":
+        specs = [W.tgv(n, 61, nu=nu, u0=0.1, amp2=0.01) for n, nu in ((33, 0.01), (33, 0.3), (33, 0.04))]
+    else:
+        bc = "bouzidi" if kind == "bouzidi" else "halfway"
+        io = "interpolated" if kind == "interpolated" else "face"
+        specs = [replace(W.channel(5, u_mean=u, steps=61, steady_tol=0.0, bc=bc, inout=io),
+                         ramp_steps=int(kind[4:]) if kind.startswith("ramp") else 20) for u in (0.04, 0.07)]
+    got = _run(ens, specs, "f64", fields_dtype="f64", qoi_every=1, series=True)
+    ref = olbm.run([oracle_case(s, qoi_every=1) for s in specs])
+    for i, r in enumerate(ref):
+        assert got["qoi"][i, U.UQLB_QOI_STATUS] == 0
+        assert rel_l2(got["fields"][i, :-1], oracle_row(r)[:-1]) < 4 * 2.7e-13, (kind, i)
