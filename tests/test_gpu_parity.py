@@ -1251,8 +1251,47 @@ def test_fp64_collision_in_fast_flows(ens, kind):
         io = "interpolated" if kind == "interpolated" else "face"
         specs = [replace(W.channel(5, u_mean=u, steps=61, steady_tol=0.0, bc=bc, inout=io),
                          ramp_steps=int(kind[4:]) if kind.startswith("ramp") else 20) for u in (0.04, 0.07)]
-    got = _run(ens, specs, "f64", fields_dtype="f64", qoi_every=1, series=True)
+    got = _run(ens, specs, "f64", qoi_every=1, series=True)
     ref = olbm.run([oracle_case(s, qoi_every=1) for s in specs])
     for i, r in enumerate(ref):
         assert got["qoi"][i, U.UQLB_QOI_STATUS] == 0
         assert rel_l2(got["fields"][i, :-1], oracle_row(r)[:-1]) < 4 * 2.7e-13, (kind, i)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("sa,na,sb,nb,bins", [(1, 1, 2, 3, 1), (3, 225, 5, 961, 7), (4, 2049, 2, 2047, 4096),
+                                              (40, 5000, 20, 3001, 8192), (9, 4099, 7, 2500, 8193),
+                                              (6, 3000, 3, 3000, 1 << 20)])
+def test_w1_counts_every_speed_in_its_bin(ens, dtype, sa, na, sb, nb, bins):
+    """The binned distance against its definition in FP64 (numpy): zero speeds, speeds on bin edges, tiny and
+    huge ones outside FP32's range of squares, ties for the largest speed, both sets non-finite in places.
+    One speed in a wrong bin moves the distance by h / n; the FP64 sum of the definition rounds each of its
+    `bins` terms and the cumulative shares by 2^-53, so equality holds to 4 bins 2^-53 of the largest term's
+    scale vmax."""
+    rng = np.random.default_rng(bins + sa)
+    sets = []
+    for s, n in ((sa, na), (sb, nb)):
+        m = (0.01 * rng.standard_normal((s, 2 * n + 1))).astype(dtype)
+        m[:, : n // 3] = 0
+        m[:, n: n + n // 4] = 0
+        k = min(n, 40)
+        m[0, :k] = (np.arange(k) * 0.25 / max(bins, 4)).astype(dtype)  # speeds on edges once vmax is 0.25
+        m[0, n: n + k] = 0
+        m[0, n - 1], m[0, 2 * n - 1] = 0.15, 0.2                        # speed 0.25 up to rounding
+        if n > 100:
+            m[0, 50], m[0, n + 50] = 1e-25, 1e-30
+            m[0, 51], m[0, n + 51] = np.nan, 0
+            m[0, 52], m[0, n + 52] = 0, -np.inf
+            m[-1, n - 2], m[-1, 2 * n - 2] = 0.2, 0.15
+        sets.append((m, n))
+    (a, na_), (b, nb_) = sets
+    w1, bound, bad = ens.w1_speed(torch.from_numpy(a).cuda(), na_, torch.from_numpy(b).cuda(), nb_, bins=bins)
+    with np.errstate(invalid="ignore"):
+        sp = [np.sqrt(m[:, :n].astype(np.float64) ** 2 + m[:, n: 2 * n].astype(np.float64) ** 2).ravel() for m, n in sets]
+    fin = [s[np.isfinite(s)] for s in sp]
+    assert tuple(bad) == tuple(len(s) - len(f) for s, f in zip(sp, fin))
+    vmax = max(f.max() for f in fin)
+    cdf = [np.cumsum(np.bincount(np.clip((f * (bins / vmax)).astype(np.int64), 0, bins - 1), minlength=bins)) / len(f)
+           for f in fin]
+    assert bound == vmax / bins
+    assert abs(w1 - np.abs(cdf[0] - cdf[1]).sum() * (vmax / bins)) <= 4 * bins * 2.0 ** -53 * vmax
