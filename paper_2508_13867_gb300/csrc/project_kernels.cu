@@ -99,6 +99,135 @@ __global__ void mc_stats_kernel(const M* __restrict__ m, int64_t S, int64_t F, i
     }
 }
 
+// Monte Carlo statistics of FP32 fields in one pass and (almost) without FP64.  FP64 instructions issue at
+// 1/75 of the FP32 rate on GB300, so the two-pass FP64 loop above is bound by its five of them per value.
+// Here the deviations d = x - c from the field's first sample c are formed exactly (a sum of two FP32
+// numbers), and sum d and sum d^2 are kept as sums of three FP32 numbers with exact rounding errors
+// (Knuth's two-sum, products by FMA): about 70 bits, more than FP64 holds.  The rest,
+// var = (sum d^2 - (sum d)^2 / S) / (S - ddof), takes pairs of FP64 numbers once per field, so that the
+// cancellation of the shift costs nothing.  A field with a non-finite value, or a deviation outside
+// [1e-15, 1e15] (whose square or its rounding error would leave FP32's range), is left to FP64.
+// A block takes 32 fields, each of its eight warps every eighth sample.  Measured on 1024 samples of 2 x
+// 512^2 + 1 fields: 0.92 against 5.09 ms.
+constexpr int kMcWarps = 8;
+struct Sum3 {
+    float a, b, c;
+};
+__device__ __forceinline__ float two_sum(float& s, float x) {  // s += x; returns the rounding error
+    const float t = __fadd_rn(s, x), v = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(x, v));
+    s = t;
+    return e;
+}
+__device__ __forceinline__ void add_low(Sum3& s, float x) { s.c = __fadd_rn(s.c, two_sum(s.b, x)); }
+__device__ __forceinline__ void add(Sum3& s, float x) { add_low(s, two_sum(s.a, x)); }
+__device__ __forceinline__ void add(Sum3& s, const Sum3& x) {
+    add(s, x.a);
+    add_low(s, x.b);
+    s.c = __fadd_rn(s.c, x.c);
+}
+struct Pair64 {
+    double h, l;
+};
+__device__ __forceinline__ Pair64 quick_sum(double a, double b) {  // |a| >= |b|, or a == 0
+    const double h = a + b;
+    return {h, b - (h - a)};
+}
+__device__ __forceinline__ Pair64 to_pair(const Sum3& s) {
+    const Pair64 p = quick_sum((double)s.a, (double)s.b);
+    return quick_sum(p.h, p.l + (double)s.c);
+}
+
+__global__ void __launch_bounds__(32 * kMcWarps) mc_stats_f32_kernel(const float* __restrict__ m, int64_t S, int64_t F,
+                                                                     int64_t ld, double* mean, double* var, int ddof) {
+    __shared__ Sum3 sd[kMcWarps][32], sq[kMcWarps][32];
+    __shared__ double sx[kMcWarps][32];
+    __shared__ int bad_warps[kMcWarps];
+    const int lane = threadIdx.x, warp = threadIdx.y;
+    const int64_t f = blockIdx.x * (int64_t)32 + lane;
+    const float* col = m + (f < F ? f : F - 1);
+    const float c = __ldg(col);
+    Sum3 d{}, q{};
+    bool bad = false;
+    auto take = [&](float x) {
+        float dh = x;
+        const float dl = two_sum(dh, -c);
+        const float t = fabsf(dh);
+        bad = bad || !(t <= 1e15f) || (t < 1e-15f && t > 0.0f);
+        const float p = __fmul_rn(dh, dh), e = __fmaf_rn(dh, dh, -p);
+        add(d, dh);
+        add(q, p);
+        add_low(q, e);
+        if (__any_sync(0xffffffffu, dl != 0.0f)) {  // values within a factor of two of c give none
+            const float d2 = dh + dh, p2 = __fmul_rn(d2, dl), e2 = __fmaf_rn(d2, dl, -p2);
+            add_low(d, dl);
+            add_low(q, p2);
+            q.c = __fadd_rn(q.c, __fmaf_rn(dl, dl, e2));
+        }
+    };
+    constexpr int kAhead = 8;
+    int64_t s = warp;
+    for (; s + (kAhead - 1) * kMcWarps < S; s += kAhead * kMcWarps) {
+        float x[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) x[k] = __ldg(col + (s + k * kMcWarps) * ld);
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) take(x[k]);
+    }
+    for (; s < S; s += kMcWarps) take(__ldg(col + s * ld));
+    sd[warp][lane] = d;
+    sq[warp][lane] = q;
+    const unsigned bad_lanes = __ballot_sync(0xffffffffu, bad);
+    if (lane == 0) bad_warps[warp] = (int)bad_lanes;
+    __syncthreads();
+    unsigned any_bad = 0;
+#pragma unroll
+    for (int w = 0; w < kMcWarps; ++w) any_bad |= (unsigned)bad_warps[w];
+    if (warp == 0 && f < F && !((any_bad >> lane) & 1)) {
+        for (int w = 1; w < kMcWarps; ++w) {
+            add(d, sd[w][lane]);
+            add(q, sq[w][lane]);
+        }
+        const double n = (double)S;
+        const Pair64 D = to_pair(d), Q = to_pair(q);
+        const double md = D.h / n, mr = (fma(-md, n, D.h) + D.l) / n;  // mean of d = md + mr
+        if (mean) mean[f] = (double)c + (md + mr);
+        if (var) {
+            // T = D^2 / n = D md + D mr, as a pair; Q - T
+            const double th = D.h * md, tl = fma(D.h, md, -th) + (D.l * md + D.h * mr);
+            const double r = Q.h - th, v = r - Q.h, e = (Q.h - (r - v)) - (th + v);
+            const double ss = fmax(r + (e + (Q.l - tl)), 0.0);
+            var[f] = ddof < 0 ? ss : ((S - ddof) > 0 ? ss / (double)(S - ddof) : NAN);
+        }
+    }
+    if (any_bad == 0) return;
+    // FP64 in two passes for the fields left to it
+    const bool mine = ((any_bad >> lane) & 1) && f < F;
+    double acc = 0.0;
+    if (mine)
+        for (int64_t k = warp; k < S; k += kMcWarps) acc += (double)__ldg(col + k * ld);
+    sx[warp][lane] = acc;
+    __syncthreads();
+    double mu = 0.0;
+    for (int w = 0; w < kMcWarps; ++w) mu += sx[w][lane];
+    mu /= (double)S;
+    __syncthreads();
+    acc = 0.0;
+    if (mine)
+        for (int64_t k = warp; k < S; k += kMcWarps) {
+            const double x = (double)__ldg(col + k * ld) - mu;
+            acc = fma(x, x, acc);
+        }
+    sx[warp][lane] = acc;
+    __syncthreads();
+    if (warp == 0 && mine) {
+        double ss = 0.0;
+        for (int w = 0; w < kMcWarps; ++w) ss += sx[w][lane];
+        if (mean) mean[f] = mu;
+        if (var) var[f] = ddof < 0 ? ss : ((S - ddof) > 0 ? ss / (double)(S - ddof) : NAN);
+    }
+}
+
 // Sum factorization of the projection on a tensor Gauss-Legendre grid.  There W[k, s] is a product
 // over the input dimensions, W[k, s] = prod_q G[alpha_kq][s_q] with G[a][s] = (w_s / 2) phi_a(x_s) (the
 // 1-D probability weight times the orthonormal Legendre polynomial), so C = W M contracts one
@@ -196,7 +325,8 @@ cudaError_t launch_mc_stats(const void* M, int dtype, int64_t S, int64_t F, int6
     if (dtype == UQLB_F64)
         mc_stats_kernel<double><<<g, 256, 0, s>>>(static_cast<const double*>(M), S, F, ld, mean, var, ddof);
     else
-        mc_stats_kernel<float><<<g, 256, 0, s>>>(static_cast<const float*>(M), S, F, ld, mean, var, ddof);
+        mc_stats_f32_kernel<<<(unsigned)((F + 31) / 32), dim3(32, kMcWarps), 0, s>>>(static_cast<const float*>(M), S, F, ld,
+                                                                                     mean, var, ddof);
     return cudaGetLastError();
 }
 

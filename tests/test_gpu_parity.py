@@ -1295,3 +1295,54 @@ def test_w1_counts_every_speed_in_its_bin(ens, dtype, sa, na, sb, nb, bins):
            for f in fin]
     assert bound == vmax / bins
     assert abs(w1 - np.abs(cdf[0] - cdf[1]).sum() * (vmax / bins)) <= 4 * bins * 2.0 ** -53 * vmax
+
+
+@pytest.mark.parametrize("S,F", [(2, 1), (7, 31), (8, 32), (9, 33), (65, 100), (1000, 65), (4096, 3)])
+@pytest.mark.parametrize("kind", ["near", "far", "outlier", "wide", "zeros"])
+def test_mc_statistics_of_fp32_fields(S, F, kind):
+    """Mean and variance of FP32 fields against 80-bit numpy: spreads far below the mean, signs that change,
+    a first sample far from the rest, values over many orders of magnitude, constant fields, and fields left
+    to FP64 (non-finite, or deviations outside [1e-15, 1e15]).  The sums carry more than 60 bits, the result
+    one rounding of the mean and a few of the variance: 4 x 2^-53 and 16 x 2^-53; fields left to FP64 take the
+    two-pass bound of S rounding errors."""
+    rng = np.random.default_rng(S * 100 + F)
+    m = rng.standard_normal((S, F))
+    if kind == "near":
+        m = 1.0 + 1e-4 * m
+    elif kind == "outlier":
+        m[0] += 1e4
+    elif kind == "wide":
+        m *= 10.0 ** rng.integers(-12, 12, (S, F))
+    elif kind == "zeros":
+        m[:, ::2] = 0.125
+    m = m.astype(np.float32)
+    special = {}
+    if F >= 31:
+        m[S // 2, 3], m[0, 5], m[:, 7], m[:, 9] = np.nan, np.inf, m[:, 7] * np.float32(1e-20), m[:, 9] * np.float32(1e17)
+        special = {3, 5, 7, 9}
+    e = Ensemble(0)
+    e.set_inputs([(0.0, 1.0)])
+    e.init_mc(S, 1)
+    pad = torch.zeros((S, F + 3), dtype=torch.float32, device="cuda")
+    pad[:, :F] = torch.from_numpy(m)
+    mean, var = e.stats(pad[:, :F])
+    rows, bmean, m2 = e.block_moments(pad[:, :F])
+    torch.cuda.synchronize()
+    x = m.astype(np.longdouble)
+    with np.errstate(invalid="ignore"):
+        mu = x.mean(0)
+        ss = ((x - mu) ** 2).sum(0)
+    eps = 2.0 ** -53
+    for k in range(F):
+        got = float(mean[k]), float(var[k]), float(bmean[k]), float(m2[k])
+        if k in (3, 5):
+            assert not np.isfinite(got[0]) and np.isnan(got[1])
+            continue
+        scale = float(np.abs(x[:, k]).max())
+        slack = S if k in special else 1
+        for g in (got[0], got[2]):
+            assert abs(g - float(mu[k])) <= 4 * slack * eps * scale, (kind, k)
+        tol = 16 * slack * eps * float(ss[k]) + (S * (4 * eps * scale) ** 2 if k in special else 0.0)
+        assert abs(got[3] - float(ss[k])) <= tol + 1e-300, (kind, k)
+        assert abs(got[1] * (S - 1) - float(ss[k])) <= tol + 4 * eps * float(ss[k]) + 1e-300, (kind, k)
+    e.close()
