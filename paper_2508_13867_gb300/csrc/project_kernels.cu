@@ -5,11 +5,13 @@
 //   gPC mean / variance (Eq. gpc_mean, Eq. gpc_std):  mean = C[0, f], var = sum_{k>=1} C[k, f]^2
 //   Monte Carlo (Eq. meanMCS, Eq. varMCS):           two passes over the samples
 // All accumulation is FP64; M may be FP32 (the ensemble's field output) or FP64.
-// The contraction is [K x S] x [S x F] with K <= a few hundred and F up to ~10^6: each thread
-// owns two fields and KB coefficients, W tiles are staged in shared memory and broadcast.
+// The contraction is [K x S] x [S x F] with K <= a few hundred and F up to ~10^6.  Three forms: one input at
+// a time on tensor grids (sf_stage_kernel), over reflected samples on symmetric sample sets
+// (reflect_kernel), dense (project_kernel).
 #include <cmath>
 #include <cstdio>
 #include <mutex>
+#include <type_traits>
 
 #include "uqlb_internal.h"
 
@@ -18,55 +20,135 @@ namespace uqlb {
 namespace {
 
 constexpr int kProjThreads = 128;
-constexpr int kKB = 16;   // coefficients per block (blockIdx.y chunk)
 constexpr int kSB = 128;  // samples per shared-memory stage
-constexpr int kFPT = 2;   // fields per thread
 
-template <typename M>
+// Dense contraction, KB coefficients per block (blockIdx.y chunk) and FPT fields per thread.  FP64
+// instructions bound it (one per warp in 19 cycles of an SM), so a term block that divides K badly costs
+// in proportion: launch_project takes the KB with the least work for K (K = 35: 37 instructions
+// per sample in one block of 36 against 51 in three of 16; the conversion of a value is shared by the
+// block's terms).
+template <typename M, int KB, int FPT>
 __global__ void __launch_bounds__(kProjThreads) project_kernel(const double* __restrict__ W, int K, int S,
                                                                const M* __restrict__ m, int64_t F, int64_t ld,
                                                                double* __restrict__ C) {
-    __shared__ double sw[kKB][kSB];
-    const int k0 = blockIdx.y * kKB;
-    const int64_t f0 = ((int64_t)blockIdx.x * kProjThreads) * kFPT + threadIdx.x;
-    double acc[kFPT][kKB];
+    __shared__ double sw[KB][kSB];
+    const int k0 = blockIdx.y * KB;
+    const int64_t f0 = ((int64_t)blockIdx.x * kProjThreads) * FPT + threadIdx.x;
+    double acc[FPT][KB];
 #pragma unroll
-    for (int a = 0; a < kFPT; ++a)
+    for (int a = 0; a < FPT; ++a)
 #pragma unroll
-        for (int k = 0; k < kKB; ++k) acc[a][k] = 0.0;
+        for (int k = 0; k < KB; ++k) acc[a][k] = 0.0;
 
     for (int s0 = 0; s0 < S; s0 += kSB) {
         const int sn = min(kSB, S - s0);
-        for (int q = threadIdx.x; q < kKB * kSB; q += kProjThreads) {
+        for (int q = threadIdx.x; q < KB * kSB; q += kProjThreads) {
             const int kk = q / kSB, ss = q % kSB;
             sw[kk][ss] = (k0 + kk < K && ss < sn) ? W[(int64_t)(k0 + kk) * S + s0 + ss] : 0.0;
         }
         __syncthreads();
         for (int ss = 0; ss < sn; ++ss) {
             const M* row = m + (int64_t)(s0 + ss) * ld;
-            double v[kFPT];
+            double v[FPT];
 #pragma unroll
-            for (int a = 0; a < kFPT; ++a) {
+            for (int a = 0; a < FPT; ++a) {
                 const int64_t f = f0 + (int64_t)a * kProjThreads;
                 v[a] = f < F ? (double)row[f] : 0.0;
             }
 #pragma unroll
-            for (int k = 0; k < kKB; ++k) {
+            for (int k = 0; k < KB; ++k) {
                 const double w = sw[k][ss];
 #pragma unroll
-                for (int a = 0; a < kFPT; ++a) acc[a][k] = fma(w, v[a], acc[a][k]);
+                for (int a = 0; a < FPT; ++a) acc[a][k] = fma(w, v[a], acc[a][k]);
             }
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int a = 0; a < kFPT; ++a) {
+    for (int a = 0; a < FPT; ++a) {
         const int64_t f = f0 + (int64_t)a * kProjThreads;
         if (f >= F) continue;
 #pragma unroll
-        for (int k = 0; k < kKB; ++k)
+        for (int k = 0; k < KB; ++k)
             if (k0 + k < K) C[(int64_t)(k0 + k) * F + f] = acc[a][k];
     }
+}
+
+// Contraction over reflected samples.  A sample set that is symmetric in every input (Clenshaw-Curtis
+// Smolyak and Gauss-Legendre grids) falls into orbits of 2^m samples that differ in the signs of their m
+// nonzero reference coordinates.  The weights of a term over an orbit are equal up to the sign that its
+// odd degrees give, so with the signed sums h[p] = sum_b (-1)^(p.b) M[s_b] (m 2^m additions) an orbit adds
+// w_k h[p_k] to term k, and nothing to terms of odd degree in a zero coordinate: 549 multiply-adds and 272
+// additions per field where the dense contraction of 137 samples and 35 terms takes 4795.  Per-thread sums
+// lie in shared memory (a term's index is data).  A field with a non-finite value takes the products one
+// by one, zero weights included, as the dense contraction does.  Measured, 137 samples x 35 terms x 130051
+// fields: 0.36 against 1.66 ms dense (with the statistics).
+constexpr int kReflThreads = 128;
+template <typename M>
+__global__ void __launch_bounds__(kReflThreads) reflect_kernel(const ReflOrbit* __restrict__ orbits, int norbits,
+                                                               const ReflTerm* __restrict__ terms,
+                                                               const int* __restrict__ members, int K, int hrows,
+                                                               const M* __restrict__ m, int64_t F, int64_t ld,
+                                                               double* __restrict__ C) {
+    extern __shared__ double s_refl[];
+    double* const acc = s_refl + threadIdx.x;                       // [K][threads]
+    double* const hs = s_refl + (int64_t)K * kReflThreads + threadIdx.x;  // [hrows][threads]
+    const int64_t f = (int64_t)blockIdx.x * kReflThreads + threadIdx.x;
+    if (f >= F) return;  // no barrier below
+    for (int k = 0; k < K; ++k) acc[k * kReflThreads] = 0.0;
+    auto at = [&](int s) { return (double)m[(int64_t)s * ld + f]; };
+    bool finite = true;
+    auto orbit = [&](auto m_c, const ReflOrbit& o) {
+        constexpr int MM = decltype(m_c)::value, N = 1 << MM;
+        double v[N];
+#pragma unroll
+        for (int b = 0; b < N; ++b) v[b] = at(__ldg(members + o.member + b));
+#pragma unroll
+        for (int d = 0; d < MM; ++d)
+#pragma unroll
+            for (int b = 0; b < N; ++b)
+                if (!(b >> d & 1)) {
+                    const double x = v[b], y = v[b | 1 << d];
+                    v[b] = x + y;
+                    v[b | 1 << d] = x - y;
+                }
+        finite = finite && isfinite(v[0]);
+#pragma unroll
+        for (int b = 0; b < N; ++b) hs[b * kReflThreads] = v[b];
+        for (int q = o.term; q < o.term + o.nterms; ++q) {
+            const ReflTerm t = terms[q];
+            acc[t.k * kReflThreads] = fma(t.w, hs[t.p * kReflThreads], acc[t.k * kReflThreads]);
+        }
+    };
+    for (int i = 0; i < norbits; ++i) {
+        const ReflOrbit o = orbits[i];
+        switch (o.m) {
+            case 0: orbit(std::integral_constant<int, 0>{}, o); break;
+            case 1: orbit(std::integral_constant<int, 1>{}, o); break;
+            case 2: orbit(std::integral_constant<int, 2>{}, o); break;
+            case 3: orbit(std::integral_constant<int, 3>{}, o); break;
+            default: orbit(std::integral_constant<int, 4>{}, o); break;
+        }
+    }
+    if (!finite) {
+        for (int k = 0; k < K; ++k) acc[k * kReflThreads] = 0.0;
+        for (int i = 0; i < norbits; ++i) {
+            const ReflOrbit o = orbits[i];
+            for (int b = 0; b < 1 << o.m; ++b) {
+                const double x = at(members[o.member + b]);
+                int q = o.term;  // terms ascend in k
+                for (int k = 0; k < K; ++k) {
+                    double w = 0.0;
+                    if (q < o.term + o.nterms && terms[q].k == k) {
+                        w = (__popc(terms[q].p & b) & 1) ? -terms[q].w : terms[q].w;
+                        ++q;
+                    }
+                    acc[k * kReflThreads] = fma(w, x, acc[k * kReflThreads]);
+                }
+            }
+        }
+    }
+    for (int k = 0; k < K; ++k) C[(int64_t)k * F + f] = acc[k * kReflThreads];
 }
 
 __global__ void gpc_stats_kernel(const double* __restrict__ C, int K, int64_t F, double* mean, double* var) {
@@ -238,9 +320,40 @@ __global__ void __launch_bounds__(32 * kMcWarps) mc_stats_f32_kernel(const float
 // group (r, j'): it loads the n inputs once and accumulates the c outputs as independent chains, so
 // the FP64 pipe (a small fraction of the FP32 rate on GB300) always has several multiply-adds to
 // issue.  FP64 throughout.
+// The points of a Gauss-Legendre rule are symmetric, so G[a][n-1-q] = (-1)^a G[a][q] up to rounding: with the
+// sums and differences of opposite inputs a degree takes half the multiply-adds (n = 5, five degrees: 4
+// additions and 15 multiply-adds instead of 25; the middle input keeps its rounding-sized weight in the
+// odd degrees, so that a non-finite value reaches every coefficient).  Points and degrees are compile-time
+// (a runtime bound left the unrolled multiply-adds of 16 points and 9 degrees in the loop, predicated
+// off).  Measured on 625 samples x 131073 fields, all four stages: 1.43 against 3.88 ms (with the statistics).
 constexpr int kSfThreads = 256;
 
-template <typename TI>
+template <int N, int CNT, typename TI>
+__device__ __forceinline__ void sf_group(const TI* src, int64_t step, const double (*G)[kSfMaxPoints], double* out,
+                                         int64_t out_ld, const int* __restrict__ o) {
+    constexpr int H = N / 2;
+    double x[N], e[H > 0 ? H : 1], d[H > 0 ? H : 1];
+#pragma unroll
+    for (int q = 0; q < N; ++q) x[q] = (double)src[q * step];
+#pragma unroll
+    for (int q = 0; q < H; ++q) {
+        e[q] = x[q] + x[N - 1 - q];
+        d[q] = x[q] - x[N - 1 - q];
+    }
+    double y[CNT];
+#pragma unroll
+    for (int a = 0; a < CNT; ++a) {
+        y[a] = N % 2 == 1 ? G[a][H] * x[H] : 0.0;
+#pragma unroll
+        for (int q = 0; q < H; ++q)
+            y[a] = q == 0 && N % 2 == 0 ? G[a][q] * (a % 2 == 0 ? e[q] : d[q]) : fma(G[a][q], a % 2 == 0 ? e[q] : d[q], y[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < CNT; ++a) out[(int64_t)__ldg(o + a) * out_ld] = y[a];
+}
+
+// N: points per input (0: runtime n, the degrees one after the other).
+template <typename TI, int N>
 __global__ void __launch_bounds__(kSfThreads) sf_stage_kernel(const TI* __restrict__ in, int64_t in_ld,
                                                               double* __restrict__ out, int64_t out_ld,
                                                               int64_t groups, int jprev, int jout, int n, int p1,
@@ -249,7 +362,13 @@ __global__ void __launch_bounds__(kSfThreads) sf_stage_kernel(const TI* __restri
     __shared__ double sG[kSfMaxDegree + 1][kSfMaxPoints];
     for (int q = threadIdx.x; q < (kSfMaxDegree + 1) * kSfMaxPoints; q += kSfThreads) {
         const int a = q / kSfMaxPoints, c = q % kSfMaxPoints;
-        sG[a][c] = a < p1 && c < n ? G[a * n + c] : 0.0;
+        double g = 0.0;
+        if (a < p1 && c < n) {
+            g = G[a * n + c];
+            // both halves' weights, which differ by rounding only, as their mean
+            if (N > 0 && 2 * c + 1 != n) g = 0.5 * (g + (a % 2 == 0 ? G[a * n + n - 1 - c] : -G[a * n + n - 1 - c]));
+        }
+        sG[a][c] = g;
     }
     __syncthreads();
     const int64_t f = (int64_t)blockIdx.x * kSfThreads + threadIdx.x;
@@ -257,28 +376,96 @@ __global__ void __launch_bounds__(kSfThreads) sf_stage_kernel(const TI* __restri
     for (int64_t g = blockIdx.y; g < groups; g += gridDim.y) {
         const int64_t r = g / jprev;
         const int jp = (int)(g - r * jprev);
+        const int* o = oidx + jp * p1;
         int cnt = 0;  // admitted degrees: a prefix of 0 .. p1 - 1
-#pragma unroll
-        for (int a = 0; a <= kSfMaxDegree; ++a)
-            if (a < p1 && __ldg(oidx + jp * p1 + a) >= 0) cnt = a + 1;
-        double acc[kSfMaxDegree + 1];
-#pragma unroll
-        for (int a = 0; a <= kSfMaxDegree; ++a) acc[a] = 0.0;
+        while (cnt < p1 && __ldg(o + cnt) >= 0) ++cnt;
         const TI* src = in + ((r * n) * jprev + jp) * in_ld + f;
         const int64_t step = (int64_t)jprev * in_ld;
-#pragma unroll
-        for (int q = 0; q < kSfMaxPoints; ++q) {
-            if (q < n) {
-                const double x = (double)src[q * step];
-#pragma unroll
-                for (int a = 0; a <= kSfMaxDegree; ++a)
-                    if (a < cnt) acc[a] = fma(sG[a][q], x, acc[a]);
+        double* dst = out + (r * jout) * out_ld + f;
+        if constexpr (N > 0) {
+            switch (cnt) {
+#define UQLB_SF_CASE(C_) \
+    case C_: sf_group<N, C_>(src, step, sG, dst, out_ld, o); break;
+                UQLB_SF_CASE(1)
+                UQLB_SF_CASE(2)
+                UQLB_SF_CASE(3)
+                UQLB_SF_CASE(4)
+                UQLB_SF_CASE(5)
+                UQLB_SF_CASE(6)
+                UQLB_SF_CASE(7)
+                UQLB_SF_CASE(8)
+                UQLB_SF_CASE(9)
+#undef UQLB_SF_CASE
+            }
+        } else {
+            for (int a = 0; a < cnt; ++a) {
+                double y = 0.0;
+                for (int q = 0; q < n; ++q) y = fma(sG[a][q], (double)src[q * step], y);
+                dst[(int64_t)__ldg(o + a) * out_ld] = y;
             }
         }
-#pragma unroll
-        for (int a = 0; a <= kSfMaxDegree; ++a)
-            if (a < cnt) out[(r * jout + __ldg(oidx + jp * p1 + a)) * out_ld + f] = acc[a];
     }
+}
+static_assert(kSfMaxDegree == 8, "sf_stage_kernel has a case for each count of degrees");
+
+template <typename TI>
+void launch_sf(dim3 grid, cudaStream_t s, const TI* in, int64_t in_ld, double* out, int64_t out_ld, int64_t groups,
+               int jprev, int jout, int n, int p1, const int* oidx, const double* G, int64_t F) {
+#define UQLB_SF_POINTS(N_) \
+    case N_: \
+        sf_stage_kernel<TI, N_><<<grid, kSfThreads, 0, s>>>(in, in_ld, out, out_ld, groups, jprev, jout, n, p1, oidx, G, F); \
+        return;
+    switch (n) {
+        UQLB_SF_POINTS(2)
+        UQLB_SF_POINTS(3)
+        UQLB_SF_POINTS(4)
+        UQLB_SF_POINTS(5)
+        UQLB_SF_POINTS(6)
+        UQLB_SF_POINTS(7)
+        UQLB_SF_POINTS(8)
+        UQLB_SF_POINTS(9)
+    }
+#undef UQLB_SF_POINTS
+    sf_stage_kernel<TI, 0><<<grid, kSfThreads, 0, s>>>(in, in_ld, out, out_ld, groups, jprev, jout, n, p1, oidx, G, F);
+}
+
+template <typename M, int KB, int FPT>
+void launch_dense(const double* W, int K, int S, const M* m, int64_t F, int64_t ld, double* C, cudaStream_t s) {
+    const int64_t per_block = (int64_t)kProjThreads * FPT;
+    const dim3 grid((unsigned)((F + per_block - 1) / per_block), (unsigned)((K + KB - 1) / KB));
+    project_kernel<M, KB, FPT><<<grid, kProjThreads, 0, s>>>(W, K, S, m, F, ld, C);
+}
+template <typename M>
+void launch_dense_any(const double* W, int K, int S, const M* m, int64_t F, int64_t ld, double* C, cudaStream_t s) {
+    // FP64 instructions per field and sample of a block size: its terms and one conversion, per block
+    constexpr int kSizes[] = {6, 12, 16, 24, 36};
+    int best = 0, cost = 0;
+    for (int kb : kSizes) {
+        const int c = (K + kb - 1) / kb * (kb + 1);
+        if (best == 0 || c < cost) {
+            best = kb;
+            cost = c;
+        }
+    }
+    switch (best) {
+        case 6: return launch_dense<M, 6, 2>(W, K, S, m, F, ld, C, s);
+        case 12: return launch_dense<M, 12, 2>(W, K, S, m, F, ld, C, s);
+        case 16: return launch_dense<M, 16, 2>(W, K, S, m, F, ld, C, s);
+        case 24: return launch_dense<M, 24, 1>(W, K, S, m, F, ld, C, s);
+        default: return launch_dense<M, 36, 1>(W, K, S, m, F, ld, C, s);
+    }
+}
+
+template <typename M>
+cudaError_t launch_refl(const ReflPlanView& p, int K, const M* m, int64_t F, int64_t ld, double* C, cudaStream_t s) {
+    const int hrows = 1 << p.max_m;
+    const size_t smem = (size_t)(K + hrows) * kReflThreads * sizeof(double);
+    static const cudaError_t opt_in = cudaFuncSetAttribute(reflect_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           kReflMaxRows * kReflThreads * (int)sizeof(double));
+    if (opt_in != cudaSuccess) return opt_in;
+    reflect_kernel<M><<<(unsigned)((F + kReflThreads - 1) / kReflThreads), kReflThreads, smem, s>>>(
+        p.orbits, p.norbits, p.terms, p.members, K, hrows, m, F, ld, C);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -288,26 +475,33 @@ cudaError_t launch_sf_stage(const void* in, int in_dtype, int64_t in_ld, double*
                             cudaStream_t s) {
     if (F <= 0 || groups <= 0) return cudaSuccess;
     if (n < 1 || n > kSfMaxPoints || p1 < 1 || p1 > kSfMaxDegree + 1) return cudaErrorInvalidValue;
-    dim3 grid((unsigned)((F + kSfThreads - 1) / kSfThreads), (unsigned)(groups < 65535 ? groups : 65535));
+    // enough blocks to fill the chip several times; a block keeps its table for all its groups
+    const int64_t gx = (F + kSfThreads - 1) / kSfThreads;
+    int64_t gy = (16 * 152 + gx - 1) / gx;
+    gy = gy < groups ? gy : groups;
+    const dim3 grid((unsigned)gx, (unsigned)(gy < 65535 ? gy : 65535));
     if (in_dtype == UQLB_F64)
-        sf_stage_kernel<double><<<grid, kSfThreads, 0, s>>>(static_cast<const double*>(in), in_ld, out, out_ld, groups,
-                                                            jprev, jout, n, p1, oidx, G, F);
+        launch_sf(grid, s, static_cast<const double*>(in), in_ld, out, out_ld, groups, jprev, jout, n, p1, oidx, G, F);
     else
-        sf_stage_kernel<float><<<grid, kSfThreads, 0, s>>>(static_cast<const float*>(in), in_ld, out, out_ld, groups,
-                                                           jprev, jout, n, p1, oidx, G, F);
+        launch_sf(grid, s, static_cast<const float*>(in), in_ld, out, out_ld, groups, jprev, jout, n, p1, oidx, G, F);
     return cudaGetLastError();
 }
 
 cudaError_t launch_project(const double* W, int K, int S, const void* M, int dtype, int64_t F, int64_t ld,
                            double* C, cudaStream_t s) {
     if (F <= 0 || K <= 0) return cudaSuccess;
-    const int64_t per_block = (int64_t)kProjThreads * kFPT;
-    dim3 grid((unsigned)((F + per_block - 1) / per_block), (unsigned)((K + kKB - 1) / kKB));
     if (dtype == UQLB_F64)
-        project_kernel<double><<<grid, kProjThreads, 0, s>>>(W, K, S, static_cast<const double*>(M), F, ld, C);
+        launch_dense_any(W, K, S, static_cast<const double*>(M), F, ld, C, s);
     else
-        project_kernel<float><<<grid, kProjThreads, 0, s>>>(W, K, S, static_cast<const float*>(M), F, ld, C);
+        launch_dense_any(W, K, S, static_cast<const float*>(M), F, ld, C, s);
     return cudaGetLastError();
+}
+
+cudaError_t launch_reflect(const ReflPlanView& p, int K, const void* M, int dtype, int64_t F, int64_t ld, double* C,
+                           cudaStream_t s) {
+    if (F <= 0 || K <= 0) return cudaSuccess;
+    return dtype == UQLB_F64 ? launch_refl(p, K, static_cast<const double*>(M), F, ld, C, s)
+                             : launch_refl(p, K, static_cast<const float*>(M), F, ld, C, s);
 }
 
 cudaError_t launch_gpc_stats(const double* C, int K, int64_t F, double* mean, double* var, cudaStream_t s) {

@@ -60,6 +60,12 @@ struct uqlb_ctx {
         std::vector<unsigned char> tables;
         int64_t rows_a = 0, rows_b = 0;
     } sf;
+    // Contraction over reflected samples (norbits = 0: not available): orbits, terms and sample indices
+    struct ReflPlan {
+        int norbits = 0, max_m = 0;
+        size_t terms_at = 0, members_at = 0;  // byte offsets into tables (orbits first)
+        std::vector<unsigned char> tables;
+    } refl;
     cudaStream_t capture_stream = nullptr;
     cudaStream_t side_stream = nullptr;           // CHANNEL groups of a grouped batch (high priority)
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
@@ -1435,6 +1441,85 @@ void build_sum_factor_plan(uqlb_ctx* ctx, int n, const std::vector<double>& gx, 
     P.p1 = p1;
 }
 
+// Orbits of the sample set under sign changes of the reference coordinates, with the terms' weights.  No
+// plan where an orbit is not complete, its weights are not equal up to the terms' parities (1e-13 of the
+// term's largest), a sample has more than kReflMaxDims nonzero coordinates, or the tables would not fit
+// the workspace of the weight matrix.
+void build_reflection_plan(uqlb_ctx* ctx) {
+    const int d = ctx->dim, K = ctx->K;
+    const int64_t S = ctx->S;
+    if (K + (1 << std::min(d, kReflMaxDims)) > kReflMaxRows || S > (1 << 20)) return;
+    std::vector<double> top(K, 0.0);
+    for (int k = 0; k < K; ++k)
+        for (int64_t s = 0; s < S; ++s) top[k] = std::max(top[k], std::fabs(ctx->W[(size_t)k * S + s]));
+    std::map<std::vector<int64_t>, std::vector<int64_t>> orbits;  // rounded |xi| -> samples
+    auto zero = [](double x) { return std::fabs(x) < 1e-12; };
+    for (int64_t s = 0; s < S; ++s) {
+        std::vector<int64_t> key(d);
+        for (int q = 0; q < d; ++q) key[q] = std::llround(std::fabs(ctx->xi[(size_t)s * d + q]) * 1e10);
+        orbits[key].push_back(s);
+    }
+    std::vector<ReflOrbit> ob;
+    std::vector<ReflTerm> terms;
+    std::vector<int32_t> members;
+    int max_m = 0;
+    for (auto& kv : orbits) {
+        const auto& list = kv.second;
+        std::vector<int> act;
+        for (int q = 0; q < d; ++q)
+            if (!zero(ctx->xi[(size_t)list[0] * d + q])) act.push_back(q);
+        const int m = (int)act.size();
+        if (m > kReflMaxDims || (int64_t)list.size() != (int64_t)1 << m) return;
+        std::vector<int32_t> at((size_t)1 << m, -1);
+        for (int64_t s : list) {
+            int b = 0;
+            for (int q = 0; q < m; ++q) b |= (ctx->xi[(size_t)s * d + act[q]] < 0.0) << q;
+            at[b] = (int32_t)s;
+        }
+        for (int32_t s : at)
+            if (s < 0) return;
+        ReflOrbit o{m, (int32_t)members.size(), (int32_t)terms.size(), 0};
+        for (int k = 0; k < K; ++k) {
+            int p = 0;
+            for (int q = 0; q < m; ++q) p |= (ctx->alpha[(size_t)k * d + act[q]] & 1) << q;
+            bool odd_at_zero = false;
+            for (int q = 0, i = 0; q < d; ++q) {
+                if (i < m && act[i] == q)
+                    ++i;
+                else
+                    odd_at_zero = odd_at_zero || (ctx->alpha[(size_t)k * d + q] & 1);
+            }
+            double w = 0.0;
+            for (int b = 0; b < 1 << m; ++b) {
+                const double v = ctx->W[(size_t)k * S + at[b]];
+                w += (__builtin_popcount(p & b) & 1) ? -v : v;
+            }
+            w = odd_at_zero ? 0.0 : w / (double)(1 << m);
+            for (int b = 0; b < 1 << m; ++b) {
+                const double v = ctx->W[(size_t)k * S + at[b]];
+                if (std::fabs(v - ((__builtin_popcount(p & b) & 1) ? -w : w)) > 1e-13 * top[k]) return;
+            }
+            if (odd_at_zero) continue;
+            terms.push_back({w, k, p});
+            ++o.nterms;
+        }
+        members.insert(members.end(), at.begin(), at.end());
+        ob.push_back(o);
+        max_m = std::max(max_m, m);
+    }
+    auto& P = ctx->refl;
+    P.terms_at = align_up(ob.size() * sizeof(ReflOrbit), 16);
+    P.members_at = P.terms_at + terms.size() * sizeof(ReflTerm);
+    const size_t total = P.members_at + members.size() * sizeof(int32_t);
+    if (total > align_up((size_t)K * S * sizeof(double), 256)) return;
+    P.tables.assign(total, 0);
+    std::memcpy(P.tables.data(), ob.data(), ob.size() * sizeof(ReflOrbit));
+    std::memcpy(P.tables.data() + P.terms_at, terms.data(), terms.size() * sizeof(ReflTerm));
+    std::memcpy(P.tables.data() + P.members_at, members.data(), members.size() * sizeof(int32_t));
+    P.max_m = max_m;
+    P.norbits = (int)ob.size();
+}
+
 // Row stride (doubles) of the sum-factorization buffers, and their workspace for F fields.
 int64_t sf_ld(int64_t F) { return (F + 31) / 32 * 32; }
 size_t sf_workspace(const uqlb_ctx* ctx, int64_t F) {
@@ -1447,6 +1532,7 @@ bool sf_available(const uqlb_ctx* ctx) { return ctx->method == UQLB_METHOD_GPC &
 int uqlb_init_gpc(uqlb_ctx* ctx, int order, int pts_per_dim, int basis, int quad) {
     if (!ctx) return set_err(nullptr, UQLB_ERR_ARG, "null context");
     ctx->sf = uqlb_ctx::SumFactorPlan{};
+    ctx->refl = uqlb_ctx::ReflPlan{};
     if (ctx->dim < 1) return set_err(ctx, UQLB_ERR_STATE, "init_gpc: call uqlb_set_inputs first");
     if (quad != UQLB_QUAD_GAUSS_LEGENDRE_TENSOR && quad != UQLB_QUAD_CLENSHAW_CURTIS_SMOLYAK)
         return set_err(ctx, UQLB_ERR_ARG, "init_gpc: unknown quadrature");
@@ -1515,6 +1601,7 @@ int uqlb_init_gpc(uqlb_ctx* ctx, int order, int pts_per_dim, int basis, int quad
     ctx->basis = basis;
     ctx->method = UQLB_METHOD_GPC;
     if (quad == UQLB_QUAD_GAUSS_LEGENDRE_TENSOR) build_sum_factor_plan(ctx, pts_per_dim, gx, gw);
+    if (!sf_available(ctx)) build_reflection_plan(ctx);
     return 0;
 }
 
@@ -2116,6 +2203,17 @@ int uqlb_project(uqlb_ctx* ctx, const void* m_dev, int dtype, int64_t n_fields, 
     size_t need = 0;
     uqlb_post_workspace_bytes(ctx, &need);
     if (workspace_bytes < need) return set_err(ctx, UQLB_ERR_OOM, "project: workspace of %zu bytes, need %zu", workspace_bytes, need);
+    if (ctx->refl.norbits > 0 && reinterpret_cast<uintptr_t>(workspace_dev) % 16 == 0) {
+        const auto& P = ctx->refl;
+        const char* ws = static_cast<const char*>(workspace_dev);
+        e = cudaMemcpyAsync(workspace_dev, P.tables.data(), P.tables.size(), cudaMemcpyHostToDevice, s);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "project: table upload");
+        const ReflPlanView v{reinterpret_cast<const ReflOrbit*>(ws), reinterpret_cast<const ReflTerm*>(ws + P.terms_at),
+                             reinterpret_cast<const int*>(ws + P.members_at), P.norbits, P.max_m};
+        e = launch_reflect(v, ctx->K, m_dev, dtype, n_fields, m_ld, coeffs_dev, s);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "project: launch");
+        return 0;
+    }
     e = cudaMemcpyAsync(workspace_dev, ctx->W.data(), ctx->W.size() * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "project: W upload");
     e = launch_project(static_cast<const double*>(workspace_dev), ctx->K, (int)ctx->S, m_dev, dtype, n_fields, m_ld,

@@ -275,6 +275,27 @@ constexpr int kSfMaxDegree = 8;
 cudaError_t launch_sf_stage(const void* in, int in_dtype, int64_t in_ld, double* out, int64_t out_ld, int64_t groups,
                             int jprev, int jout, int n, int p1, const int* oidx, const double* G, int64_t F,
                             cudaStream_t s);
+// Contraction over reflected samples (project_kernels.cu): orbits of 2^m samples (their indices at
+// members[member ..], bit d of the position: the sign of the orbit's d-th nonzero coordinate), each with its
+// terms k (ascending), their weight w on the all-positive sample and the parities p of their degrees in the
+// nonzero coordinates.
+struct ReflOrbit {
+    int32_t m, member, term, nterms;
+};
+struct alignas(16) ReflTerm {
+    double w;
+    int32_t k, p;
+};
+struct ReflPlanView {
+    const ReflOrbit* orbits;
+    const ReflTerm* terms;
+    const int* members;
+    int norbits, max_m;
+};
+constexpr int kReflMaxDims = 4;    // nonzero coordinates of a sample
+constexpr int kReflMaxRows = 128;  // K + 2^m rows of per-thread values in shared memory
+cudaError_t launch_reflect(const ReflPlanView& p, int K, const void* M, int dtype, int64_t F, int64_t ld, double* C,
+                           cudaStream_t s);
 cudaError_t launch_project(const double* W, int K, int S, const void* M, int dtype,
                            int64_t F, int64_t ld, double* C, cudaStream_t s);
 cudaError_t launch_gpc_stats(const double* C, int K, int64_t F, double* mean, double* var,

@@ -1346,3 +1346,56 @@ def test_mc_statistics_of_fp32_fields(S, F, kind):
         assert abs(got[3] - float(ss[k])) <= tol + 1e-300, (kind, k)
         assert abs(got[1] * (S - 1) - float(ss[k])) <= tol + 4 * eps * float(ss[k]) + 1e-300, (kind, k)
     e.close()
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("dim,order,pts,quad", [(1, 0, 1, 0), (1, 8, 9, 0), (1, 3, 2, 0), (2, 5, 7, 0), (3, 4, 5, 0),
+                                                (4, 4, 5, 0), (2, 8, 16, 0), (3, 2, 4, 0), (2, 4, 10, 0), (5, 2, 3, 0),
+                                                (2, 3, 0, 1), (3, 3, 3, 1), (4, 3, 3, 1), (4, 4, 3, 1), (2, 2, 5, 1),
+                                                (5, 2, 2, 1)])
+@pytest.mark.parametrize("F", [1, 129, 257])
+def test_projection_contractions(dtype, dim, order, pts, quad, F):
+    """Every form of the projection (one input at a time with compile-time and runtime points, over reflected
+    samples, dense in blocks of terms) against W M in 80-bit numpy: S products and sums of at most |W| |M|
+    each rounded, S 2^-53 sum |W| |M| (twice: the forms' weights differ from W by rounding).  A field with a
+    NaN in one sample is NaN in every coefficient."""
+    e = Ensemble(0)
+    e.set_inputs([(-1.0, 1.0)] * dim)
+    U.uqlb_init_gpc(e.ctx, order, pts, 0, quad)
+    S, K = e.num_samples, e.num_terms
+    Wm = U.uqlb_get_weight_matrix(e.ctx).astype(np.longdouble)
+    m = W.random_fields(S, F, seed=S + F, dtype=dtype)
+    m[:, 0] *= 1e6
+    ref = np.empty((K, F), dtype=np.longdouble)
+    for k in range(K):
+        ref[k] = (Wm[k][:, None] * m).sum(0)
+    bound = 2 * max(S, 8) * 2.0 ** -53 * (np.abs(Wm) @ np.abs(m.astype(np.longdouble))) + 1e-300
+    if F > 1:
+        m[S - 1, F - 1] = np.nan
+    pad = torch.zeros((S, F + 5), dtype=torch.float32 if dtype == np.float32 else torch.float64, device="cuda")
+    pad[:, :F] = torch.from_numpy(m)
+    mt = pad[:, :F]
+    code = U.UQLB_F32 if dtype == np.float32 else U.UQLB_F64
+    out = [e.project(mt)]
+    small = torch.empty(U.uqlb_post_workspace_bytes(e.ctx), dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    for form in ("small", "noalloc", "block"):
+        c = torch.full((K, F), 7.0, dtype=torch.float64, device="cuda")
+        if form == "small":
+            U.uqlb_project(e.ctx, mt.data_ptr(), code, F, F + 5, c.data_ptr(), small.data_ptr(), small.numel(), stream)
+        elif form == "noalloc":
+            if K * S > 131072:
+                continue
+            U.uqlb_project_noalloc(e.ctx, mt.data_ptr(), code, F, F + 5, c.data_ptr(), stream)
+        else:
+            U.uqlb_project_block(e.ctx, mt.data_ptr(), code, F, F + 5, 0, S, c.data_ptr(), small.data_ptr(),
+                                 small.numel(), stream)
+        out.append(c)
+    torch.cuda.synchronize()
+    for c in out:
+        got = c.cpu().numpy()
+        good = F - 1 if F > 1 else F
+        assert np.all(np.abs(got[:, :good] - ref[:, :good]) <= bound[:, :good])
+        if F > 1:
+            assert np.isnan(got[:, F - 1]).all()
+    e.close()
