@@ -481,9 +481,10 @@ void strip_lanes(int nx, int64_t n, int* T, int* G, int* closed) {
     }
 }
 
-// ids: the caller's index of each sample (the output row), nullptr for 0..n-1.
+// ids: the caller's index of each sample (the output row), nullptr for 0..n-1.  sizes_only: the obstacle
+// masks stay empty (of their full size), for the workspace query, which plans every tile geometry.
 int plan_batch(const uqlb_sample* smp, int64_t n, const uqlb_run_opts* o, BatchPlan& P, std::string& why,
-               const TuneChoice& tuned = TuneChoice(), const int64_t* ids = nullptr) {
+               const TuneChoice& tuned = TuneChoice(), const int64_t* ids = nullptr, bool sizes_only = false) {
     if (n <= 0 || n > (1 << 24)) {
         why = "sample count out of range";
         return UQLB_ERR_ARG;
@@ -681,7 +682,7 @@ int plan_batch(const uqlb_sample* smp, int64_t n, const uqlb_run_opts* o, BatchP
                 d.mask_off = (int32_t)P.masks.size();
                 P.masks.resize(P.masks.size() + (size_t)mask_words(d) * s.ny, 0u);
                 uint32_t* m = P.masks.data() + d.mask_off;
-                for (int y = 0; y < s.ny; ++y)
+                for (int y = 0; y < s.ny && !sizes_only; ++y)
                     for (int x = 0; x < s.nx; ++x)
                         if (sample_solid(s, x, y)) m[(size_t)y * mask_words(d) + (x >> 5)] |= 1u << (x & 31);
             }
@@ -1049,7 +1050,7 @@ int batch_bytes(const uqlb_sample* samples, int64_t n, const uqlb_run_opts* opts
 }
 int batch_bytes_one(const uqlb_sample* samples, int64_t n, const uqlb_run_opts* opts, size_t* bytes, std::string& why) {
     BatchPlan P;
-    if (int rc = plan_batch(samples, n, opts, P, why)) return rc;
+    if (int rc = plan_batch(samples, n, opts, P, why, TuneChoice(), nullptr, true)) return rc;
     size_t best = P.total;
     if (opts->tile_rows == 0 && opts->nodes_per_thread == 0) {
         for (int r : kGeomRows)
@@ -1059,7 +1060,7 @@ int batch_bytes_one(const uqlb_sample* samples, int64_t n, const uqlb_run_opts* 
                 o.nodes_per_thread = q;
                 BatchPlan Q;
                 std::string ignore;
-                if (plan_batch(samples, n, &o, Q, ignore) == 0) best = std::max(best, Q.total);
+                if (plan_batch(samples, n, &o, Q, ignore, TuneChoice(), nullptr, true) == 0) best = std::max(best, Q.total);
             }
     }
     *bytes = best;
