@@ -208,8 +208,10 @@ __device__ __forceinline__ void bgk(C g[9], C omega, C drho, C jx, C jy, C ux, C
 #pragma unroll
     for (int i : {1, 2, 5, 6}) {
         const int o = opp(i);
-        const C cj = C(cx(i)) * jx + C(cy(i)) * jy;
-        const C cu = C(cx(i)) * ux + C(cy(i)) * uy;
+        // (not C(cx(i)) * jx + C(cy(i)) * jy: the compiler keeps a product with zero, which is not zero for
+        // infinities)
+        const C cj = i == 1 ? jx : (i == 2 ? jy : (i == 5 ? jx + jy : jy - jx));
+        const C cu = i == 1 ? ux : (i == 2 ? uy : (i == 5 ? ux + uy : uy - ux));
         const C A = wgt<C>(i) * (drho + C(4.5) * cj * cu - ju15);
         const C gi = fma(lin<C>(i), cj, A);
         const C go = fma(-lin<C>(i), cj, A);

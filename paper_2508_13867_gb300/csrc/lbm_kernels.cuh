@@ -104,6 +104,26 @@ __device__ __forceinline__ C inflow(const SampleDev& sp, C yy, int t) {
     return C(4) * C(sp.uin_max) * ramp * yy * (H - yy) / (H * H);
 }
 
+// The FP32 terms of inflow<float>() that do not depend on the node, with its roundings: 4 u_max, the
+// ramp's length and the step from which it is 1 (t < ramp_steps in integers), H and H H.  The record
+// holds FP64; a conversion or comparison per direction and step put some thousand cycles of FP64
+// latency on the block that holds the inlet, which the whole cluster waits for.
+struct Inflow32 {
+    float u4, ramp_len, H, HH;
+    int ramp_end;
+    __device__ explicit Inflow32(const SampleDev& sp)
+        : u4(4.0f * (float)sp.uin_max),
+          ramp_len((float)sp.ramp_steps),
+          H((float)sp.ny),
+          HH(H * H),
+          ramp_end(sp.ramp_steps > 0.0 ? (int)fmin(ceil(sp.ramp_steps), 2147483647.0) : 0) {}
+    // 4 u_max times the ramp at step t
+    __device__ __forceinline__ float factor(int t) const {
+        return t < ramp_end ? u4 * (0.5f * (1.0f - cospif((float)t / ramp_len))) : u4;
+    }
+    __device__ __forceinline__ float at(float factor, float yy) const { return factor * yy * (H - yy) / HH; }
+};
+
 // The same in FP64 split for the three directions of an inlet node: the factor of the profile, once per
 // node and step (its cosine and divisions are some fifty FP64 instructions, on the warps that every
 // step waits for), and the profile at y + (1 - cy)/2.
@@ -663,9 +683,18 @@ __device__ __forceinline__ void process_tile(const KParams& p, int t, int tile, 
 template <int NT>
 __device__ __forceinline__ void step_extent(const KParams& p, int t, TileShared<NT>& sh) {
     if (threadIdx.x == 0 && threadIdx.y == 0) {
-        const int nact = active_samples(p, t);
-        sh.nact = nact;
-        sh.ntiles = nact > 0 ? p.samples[nact - 1].tile_base + p.samples[nact - 1].tiles : 0;
+        // Mostly every sample still runs (the table is ordered by descending steps).  The loads of that
+        // case do not depend on one another; the search is a chain of log2(n) of them, more than a
+        // microsecond of a small batch's step.
+        const int n = p.nsamples, tiles = p.samples[n - 1].tile_base + p.samples[n - 1].tiles;
+        if (p.steps_sorted[n - 1] > t) {
+            sh.nact = n;
+            sh.ntiles = tiles;
+        } else {
+            const int nact = active_samples(p, t);
+            sh.nact = nact;
+            sh.ntiles = nact > 0 ? p.samples[nact - 1].tile_base + p.samples[nact - 1].tiles : 0;
+        }
     }
     __syncthreads();
 }
@@ -1609,15 +1638,6 @@ __host__ __device__ constexpr size_t cluster_state_bytes(int rw, int ny, int eb)
 template <typename S>
 constexpr int cluster_bank_span = 128 / (int)sizeof(S);
 
-// The cluster kernel's node pass: one copy per step parity (compile-time parity) or one copy with the
-// parity tested per population.  UQLB_CLUSTER_SPLIT_PARITY 1: split, 0: not, 2: split for 16-bit
-// storage only.  Measured (GLUPS, split / not): FP32 cylinder 56.1 / 57.9, BF16 channel samples of the
-// uneven batch 57.4 / 53.6.
-#ifndef UQLB_CLUSTER_SPLIT_PARITY
-#define UQLB_CLUSTER_SPLIT_PARITY 2
-#endif
-template <typename S>
-constexpr bool kClusterSplitParity = UQLB_CLUSTER_SPLIT_PARITY == 1 || (UQLB_CLUSTER_SPLIT_PARITY == 2 && sizeof(S) == 2);
 template <typename S, int CW>
 __global__ void __launch_bounds__(kClusterThreads, 1) cluster_kernel(KParams p) {
     extern __shared__ __align__(16) unsigned char s6_raw[];
@@ -1683,6 +1703,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) cluster_kernel(KParams p) 
     const C omega = (C)sp.omega;
     const bool sr = sizeof(S) == 2 && p.stochastic != 0;
     const uint32_t sid = (uint32_t)sp.sample_id;
+    const Inflow32 inlet(sp);
     // The fluid nodes in four lists, each in row-major order: boundary nodes (a link that is not
     // interior: boundary rules), interior nodes at the slab's left and at its right edge (three
     // neighbours in the next slab) and the rest (every neighbour in this slab), so that a warp
@@ -1766,99 +1787,11 @@ __global__ void __launch_bounds__(kClusterThreads, 1) cluster_kernel(KParams p) 
         // work units of 32 list entries, one per lane: warp w takes unit w in the first round and unit
         // 32 r + 31 - w in round r >= 1.  The lists start with the costlier boundary and edge nodes,
         // so the warps that took those in the first round take no unit of a last, partial round.
-        if constexpr (kClusterSplitParity<S>) {
-            // the parity of the step is a compile-time branch of the node pass (one copy of the pass per
-            // parity), so no per-population test of it remains
-            auto node_pass = [&](auto parity) {
-                constexpr bool ODD = decltype(parity)::value;
-                const int lane = tid & 31, wid = tid >> 5;
-                constexpr int NW = kClusterThreads / 32;
-                for (int r = 0; r * NW * 32 < e3; ++r) {
-                    const int k = (r * NW + (r == 0 ? wid : NW - 1 - wid)) * 32 + lane;
-                    if (k >= e3) continue;
-                    const uint32_t e = list[k];
-                    const int yn = (int)(e >> 16), xn = (int)(e & 0xFFFFu), own = yn * RW + xn;
-                    const uint32_t lw = k < e0 ? links[yn * RC + xn] : 0u;
-                    C g[9];
-                    if constexpr (ODD) {
-                        S v[9];
-                        gather_odd(k, yn, xn, own, lw, v);
-#pragma unroll
-                        for (int i = 0; i < 9; ++i) g[i] = Storage<S>::load(v + i, qz, i);
-        
-        } else {
-#pragma unroll
-                        for (int i = 0; i < 9; ++i) g[i] = Storage<S>::load(lat + own + i * RC, qz, i);
-                    }
-                    C drho, jx, jy, ux, uy;
-                    moments(g, drho, jx, jy, ux, uy);
-                    bgk(g, omega, drho, jx, jy, ux, uy);
-                    const uint32_t h = sr ? mix32((uint32_t)((int64_t)yn * sp.pitch + x0 + xn) * 0x9E3779B1u +
-                                                  (uint32_t)t * 0x85EBCA77u + sid * 0xC2B2AE3Du)
-                                          : 0u;
-                    // the stored value of population i (rounded as the storage rounds)
-                    auto cvt = [&](C v, int i) {
-                        S r;
-                        if (sr)
-                            Storage<S>::store_sr(&r, v, (h * (0x2545F491u + 0x6A09E668u * (uint32_t)i)) >> 16, qz, i);
-                        else
-                            Storage<S>::store(&r, v, qz, i);
-                        return r;
-                    };
-                    if (k >= e0) {
-                        // every link interior: even steps write g*_i into the node's slot opp(i), odd steps
-                        // into slot i of the neighbour x + c_i (across the slab's edge for the three
-                        // populations of an edge node that leave it)
-                        lat[own] = cvt(g[0], 0);
-                        const bool edge = k < e2, at_left = k < e1;
-#pragma unroll
-                        for (int i = 1; i < 9; ++i) {
-                            if constexpr (!ODD)
-                                lat[own + opp(i) * RC] = cvt(g[i], i);
-                            else if (edge && (at_left ? cx(i) < 0 : cx(i) > 0))
-                                st_cluster<S>(remote(at_left, i, yn + cy(i)), cvt(g[i], i));
-                            else
-                                lat[own + i * RC + cy(i) * RW + cx(i)] = cvt(g[i], i);
-                        }
-                        continue;
-                    }
-                    lat[own] = cvt(g[0], 0);
-#pragma unroll
-                    for (int i = 1; i < 9; ++i) {
-                        const int cls = (lw >> (3 * i)) & 7;
-                        const int o = opp(i);
-                        if (cls == kInterior) {
-                            if constexpr (!ODD) {
-                                lat[own + o * RC] = cvt(g[i], i);
-                            } else {
-                                const int dl = xn + cx(i), dy = yn + cy(i);
-                                if (dl >= 0 && dl < ncol)
-                                    lat[dy * RW + i * RC + dl] = cvt(g[i], i);
-                                else
-                                    st_cluster<S>(remote(dl < 0, i, dy), cvt(g[i], i));
-                            }
-                        } else if (cls == kWall || cls == kSolid) {
-                            lat[own + o * RC] = cvt(g[i], i);
-                            if (f_step && cls == kSolid) {
-                                const C fs = g[i] + wgt<C>(i);
-                                fx += (double)(C(2 * cx(i)) * fs);
-                                fy += (double)(C(2 * cy(i)) * fs);
-                            }
-                        } else if (cls == kInlet) {
-                            const C yy = C(yn) + C(0.5) - C(0.5) * C(cy(o));
-                            lat[own + o * RC] = cvt(g[i] + C(6) * wgt<C>(o) * C(cx(o)) * inflow<C>(sp, yy, t), i);
-                        } else {
-                            const C cu = C(cx(o)) * ux + C(cy(o)) * uy;
-                            lat[own + o * RC] = cvt(-g[i] + wgt<C>(o) * (C(9) * cu * cu - C(3) * (ux * ux + uy * uy)), i);
-                        }
-                    }
-                }
-            };
-            if (odd)
-                node_pass(std::true_type{});
-            else
-                node_pass(std::false_type{});
-            } else {
+        // One copy of the node pass per parity of the step, so that no test of it remains per population:
+        // FP32 cylinder 5.10 against 5.44 us per step with the test, BF16 channel samples of the uneven
+        // batch 57.4 against 53.6 GLUPS.
+        auto node_pass = [&](auto parity) {
+            constexpr bool ODD = decltype(parity)::value;
             const int lane = tid & 31, wid = tid >> 5;
             constexpr int NW = kClusterThreads / 32;
             for (int r = 0; r * NW * 32 < e3; ++r) {
@@ -1868,12 +1801,13 @@ __global__ void __launch_bounds__(kClusterThreads, 1) cluster_kernel(KParams p) 
                 const int yn = (int)(e >> 16), xn = (int)(e & 0xFFFFu), own = yn * RW + xn;
                 const uint32_t lw = k < e0 ? links[yn * RC + xn] : 0u;
                 C g[9];
-                if (odd) {
+                if constexpr (ODD) {
                     S v[9];
                     gather_odd(k, yn, xn, own, lw, v);
 #pragma unroll
                     for (int i = 0; i < 9; ++i) g[i] = Storage<S>::load(v + i, qz, i);
-                } else {
+    
+    } else {
 #pragma unroll
                     for (int i = 0; i < 9; ++i) g[i] = Storage<S>::load(lat + own + i * RC, qz, i);
                 }
@@ -1900,7 +1834,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) cluster_kernel(KParams p) 
                     const bool edge = k < e2, at_left = k < e1;
 #pragma unroll
                     for (int i = 1; i < 9; ++i) {
-                        if (!odd)
+                        if constexpr (!ODD)
                             lat[own + opp(i) * RC] = cvt(g[i], i);
                         else if (edge && (at_left ? cx(i) < 0 : cx(i) > 0))
                             st_cluster<S>(remote(at_left, i, yn + cy(i)), cvt(g[i], i));
@@ -1910,12 +1844,13 @@ __global__ void __launch_bounds__(kClusterThreads, 1) cluster_kernel(KParams p) 
                     continue;
                 }
                 lat[own] = cvt(g[0], 0);
+                const float in_factor = x0 + xn == 0 ? inlet.factor(t) : 0.0f;
 #pragma unroll
                 for (int i = 1; i < 9; ++i) {
                     const int cls = (lw >> (3 * i)) & 7;
                     const int o = opp(i);
                     if (cls == kInterior) {
-                        if (!odd) {
+                        if constexpr (!ODD) {
                             lat[own + o * RC] = cvt(g[i], i);
                         } else {
                             const int dl = xn + cx(i), dy = yn + cy(i);
@@ -1933,14 +1868,18 @@ __global__ void __launch_bounds__(kClusterThreads, 1) cluster_kernel(KParams p) 
                         }
                     } else if (cls == kInlet) {
                         const C yy = C(yn) + C(0.5) - C(0.5) * C(cy(o));
-                        lat[own + o * RC] = cvt(g[i] + C(6) * wgt<C>(o) * C(cx(o)) * inflow<C>(sp, yy, t), i);
+                        lat[own + o * RC] = cvt(g[i] + C(6) * wgt<C>(o) * C(cx(o)) * inlet.at(in_factor, yy), i);
                     } else {
                         const C cu = C(cx(o)) * ux + C(cy(o)) * uy;
                         lat[own + o * RC] = cvt(-g[i] + wgt<C>(o) * (C(9) * cu * cu - C(3) * (ux * ux + uy * uy)), i);
                     }
                 }
             }
-        }
+        };
+        if (odd)
+            node_pass(std::true_type{});
+        else
+            node_pass(std::false_type{});
         if (f_step) {
             double v[2] = {fx, fy};
             block_sum<2, kClusterThreads>(v, s_red);
