@@ -180,7 +180,7 @@ typedef struct {
     int32_t storage;          /* population storage: UQLB_F64, F32, F16, BF16 or FX16 (stored as f - w) */
     int32_t fields_dtype;     /* dtype of the field output M: UQLB_F64 or UQLB_F32 */
     int64_t qoi_every;        /* stride of the in-kernel QoI series (0: none) */
-    int32_t chunk_steps;      /* steps per captured CUDA graph (even, 2..1024; 0: default 64) */
+    int32_t chunk_steps;      /* steps per captured CUDA graph (even, 2..1024; 0: 32 to 96, whole graphs) */
     int32_t tile_rows;        /* rows per tile (see above; 0: tuned or default) */
     int32_t nodes_per_thread; /* nodes per thread along x (see above; 0: tuned or default) */
     int32_t rounding;         /* 16-bit storage (F16, BF16, FX16): UQLB_ROUND_AUTO (= stochastic), NEAREST or STOCHASTIC */

@@ -2621,6 +2621,31 @@ const StripBlocks& strip_regs_blocks() {
     return b;
 }
 
+// Rows per range of a launch that splits every group of samples into equal parts, 0 where equal ranges
+// over all rows are better (or heights differ).  The time of a launch in units of one phase of one warp: a
+// range of n rows takes n + 2 (NS - 1) iterations one after the other, about five units each, or the
+// work of the busiest SM, NS n + NS (NS - 1) phases of each of its blocks.  Equal ranges take the pieces of
+// two groups where they cross (2 NS (NS - 1) and 4 (NS - 1) instead).  grid: most blocks at once.
+inline int strip_part(int64_t nsup, int ny, int warps, int ns, int64_t grid) {
+    if (ny <= 0 || nsup * warps > grid * kStripWarps) return 0;
+    const int64_t sms = sm_count(), groups = grid * kStripWarps / warps;
+    auto cost = [&](int64_t blocks, int64_t n, int64_t pieces) {
+        return std::max(5 * (n + pieces * 2 * (ns - 1)), (blocks + sms - 1) / sms * (ns * n + pieces * ns * (ns - 1)));
+    };
+    const int64_t per = (nsup * ny + groups - 1) / groups;
+    int64_t best = cost(grid, per, per >= ny || ny % per != 0 ? 2 : 1);
+    int part = 0;
+    for (int64_t parts = std::min<int64_t>(groups / nsup, ny); parts >= 1; --parts) {
+        const int64_t n = (ny + parts - 1) / parts, used = (ny + n - 1) / n;
+        const int64_t c = cost((nsup * used * warps + kStripWarps - 1) / kStripWarps, n, 1);
+        if (c <= best) {
+            best = c;
+            part = (int)n;
+        }
+    }
+    return part;
+}
+
 template <typename S, int W, int D, bool ODD>
 cudaError_t launch_strip_regs_d(const KParams& p, const BatchGeometry& g, cudaStream_t s, bool prepare_only,
                                 StripBlocks* blocks) {
@@ -2641,14 +2666,21 @@ cudaError_t launch_strip_regs_d(const KParams& p, const BatchGeometry& g, cudaSt
             map.start[k.warp + 1] = (uint8_t)n;
         }
     }
-    // at most one row of a group's T samples per group of G warps
-    const int64_t rows = g.strip_ny > 0 ? (g.nsamples + g.strip_t - 1) / g.strip_t * g.strip_ny : g.total_rows;
-    const int64_t most = (rows * g.strip_g + kStripWarps - 1) / kStripWarps;
     int bps = 0, kb = 0;
     strip_launch_shape(sb, g, &bps, &kb);
+    const int64_t nsup = (g.nsamples + g.strip_t - 1) / g.strip_t;
+    const int64_t rows = g.strip_ny > 0 ? nsup * g.strip_ny : g.total_rows;
+    // at most one row of a group's T samples per group of G warps
+    const int64_t most = (rows * g.strip_g + kStripWarps - 1) / kStripWarps;
     const int64_t resident = std::max<int64_t>((int64_t)bps * sm_count(), (g.strip_g + kStripWarps - 1) / kStripWarps);
+    int64_t grid = std::min<int64_t>(std::min(most, resident), kStripMaxWarps / kStripWarps);
+    map.part = strip_part(nsup, g.strip_ny, g.strip_g, kStripSteps<S>, grid);
+    if (map.part > 0) {
+        const int64_t parts = (g.strip_ny + map.part - 1) / map.part;
+        grid = (nsup * parts * g.strip_g + kStripWarps - 1) / kStripWarps;
+    }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)std::min<int64_t>(std::min(most, resident), kStripMaxWarps / kStripWarps));
+    cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(kStripThreads);
     cfg.stream = s;
     cudaLaunchAttribute at[1];

@@ -20,7 +20,10 @@
 // alone takes five, 0.857 useful lanes against 0.8.
 //
 // Work: the rows of the running samples, T samples side by side, are split into equal ranges, one per
-// group of G warps.  A piece (range x sample) of L rows runs L + 2 (NS - 1) iterations.
+// group of G warps.  A piece (range x sample) of L rows runs L + 2 (NS - 1) iterations, so a batch with
+// fewer groups of samples than ranges splits each group into equal parts instead: no range then holds
+// parts of two (strip_part; 20 x 100^2 FP32: 2.8 us per step, equal ranges 4.1; 8 x
+// 256^2 3.6; 127^2 x 128 11.1, equal ranges 11.4).
 //
 // What bounds it (625 x 256^2 FP32, ncu): the register file's read ports.  A packed FMA of three
 // distinct registers takes three cycles (two with a reused or immediate operand, measured), about 600 of
@@ -355,11 +358,15 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
     const int nact = p.steps_sorted[p.nsamples - 1] > t ? p.nsamples : active_samples(p, t);
     const int nsup = (nact + T - 1) / T;
     const int rows = map.ny > 0 ? nsup * map.ny : p.row_base[nact];
-    const int per = (rows + ngroups - 1) / ngroups;
-    const int r1 = min(rows, (group + 1) * per);
+    // ranges: equal shares of all rows, or (small batches) `part` rows of one group of samples, so that no
+    // range holds parts of two
+    const int parts = map.part > 0 ? (map.ny + map.part - 1) / map.part : 0;
+    const int per = parts > 0 ? map.part : (rows + ngroups - 1) / ngroups;
+    const int r0 = parts > 0 ? group / parts * map.ny + group % parts * per : group * per;
+    const int r1 = parts > 0 ? min(min(rows, r0 + per), (group / parts + 1) * map.ny) : min(rows, r0 + per);
     const bool series = p.qoi_every > 0 && p.series != nullptr;
 
-    for (int r = group * per; r < r1;) {
+    for (int r = r0; r < r1;) {
         int m, rb, ny;
         if (map.ny > 0) {
             ny = map.ny;
@@ -387,7 +394,7 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
         const int sslot = __ldg(&sp->slot);
         const float omega = (float)__ldg(&sp->omega);
         const int64_t f_off = __ldg(&sp->f_off);
-        const bool second = ((p.sel[sslot] ^ ((t - t0) / NS)) & 1) != 0;
+        const bool second = ((p.sel[sslot] ^ ((t - t0) / p.spl)) & 1) != 0;
         StripPiece<S> pc;
         pc.src = static_cast<const S*>(second ? p.arena2 : p.arena) + f_off + xa;
         pc.dst = static_cast<S*>(second ? p.arena : p.arena2) + f_off + xa;
@@ -404,7 +411,7 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
         pc.sid = (uint32_t)__ldg(&sp->sample_id);
         pc.om = packed_bgk(omega);
         pc.qz = quanta_of<S>(p, j);
-        const int n_mine = have ? min(NS, steps - t) : 0;
+        const int n_mine = have ? min(p.spl, steps - t) : 0;
 
         const int n_max = __reduce_max_sync(kAll, n_mine);
         bool rec = false;
@@ -444,10 +451,11 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) part[k] += __shfl_xor_sync(kAll, part[k], o);
             }
-            const int kr = group;
+            // pieces are numbered along the ranges: a piece is one range's part of one group of samples
+            const int piece = parts > 0 ? group : m + group;
             int last = 0;
             if (lane == 0) {
-                double* to = p.kpart + ((((int64_t)(m + kr) * G + slot) * T + c) * NS);
+                double* to = p.kpart + ((((int64_t)piece * G + slot) * T + c) * NS);
 #pragma unroll
                 for (int k = 0; k < NS; ++k) to[k] = part[k];
                 __threadfence();
@@ -457,12 +465,13 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
             last = __shfl_sync(kAll, last, 0);
             if (!last) continue;
             __threadfence();
-            const int kr0 = rb / per, kr1 = (rb + ny - 1) / per;
+            const int first = parts > 0 ? m * parts : m + rb / per;
+            const int pieces = parts > 0 ? parts : (rb + ny - 1) / per - rb / per + 1;
             double acc[NS];
 #pragma unroll
             for (int k = 0; k < NS; ++k) acc[k] = 0.0;
-            for (int q = lane; q < (kr1 - kr0 + 1) * G; q += 32) {
-                const int s = q % G, at = m + kr0 + q / G;
+            for (int q = lane; q < pieces * G; q += 32) {
+                const int s = q % G, at = first + q / G;
                 if (!((warps >> s) & 1)) continue;
                 const double* from = p.kpart + ((((int64_t)at * G + s) * T + c) * NS);
 #pragma unroll
@@ -474,7 +483,7 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
                 for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(kAll, acc[k], o);
             if (lane == 0) {
                 const SampleDev* sc = p.samples + jc;
-                const int n_c = min(NS, sc->steps - t);
+                const int n_c = min(p.spl, sc->steps - t);
                 const int64_t row = (int64_t)sc->sample_id * p.series_ld;
 #pragma unroll
                 for (int k = 0; k < NS; ++k)

@@ -791,7 +791,6 @@ int plan_batch(const uqlb_sample* smp, int64_t n, const uqlb_run_opts* o, BatchP
     g.strip_ny = strips && uniform_ny ? smp[0].ny : 0;
     g.cluster = cluster ? 1 : 0;
     g.cluster_nx = g.cluster_ny = 0;
-    g.pad_ = 0;
     {
         // launch shape of the three-step strips: the caller's, else the tuned one, else the default
         const int sb = o ? o->strip_blocks_per_sm : 0, ss = o ? o->strip_stage : 0, sk = o ? o->strip_smem_kb : 0;
@@ -1067,6 +1066,25 @@ int batch_bytes_one(const uqlb_sample* samples, int64_t n, const uqlb_run_opts* 
     return 0;
 }
 
+// Steps per graph of a run of `steps` steps: a multiple of the steps per launch (even: a graph keeps the
+// parity of its first step) in 32..96.  A graph costs about four microseconds besides its steps, a launch
+// past the last step 1.5; the run takes whole graphs (272 steps at 4 per launch: 4 graphs of 68 steps
+// instead of 5 of 64 with 12 launches past the end).
+int default_chunk(int64_t steps, int spl) {
+    const int unit = spl % 2 == 0 ? spl : 2 * spl;
+    int best = 0;
+    double least = 0.0;
+    for (int c = 96 / unit * unit; c >= 32; c -= unit) {
+        const int64_t graphs = (std::max<int64_t>(steps, 1) + c - 1) / c;
+        const double cost = 4.0 * graphs + 1.5 * (double)(graphs * c - steps) / spl;
+        if (best == 0 || cost < least) {
+            best = c;
+            least = cost;
+        }
+    }
+    return best;
+}
+
 // One planned batch: tables, init (or resume), the time loop, finalize.  own_timing: the loop
 // records the context's loop events (a batch run in groups times all groups from outside).
 int run_planned(uqlb_ctx* ctx, const BatchPlan& P, int64_t n, const uqlb_run_opts* opts, void* workspace_dev,
@@ -1075,7 +1093,8 @@ int run_planned(uqlb_ctx* ctx, const BatchPlan& P, int64_t n, const uqlb_run_opt
     const bool resume = opts->start_step > 0;
     // a chunk is a whole number of launches
     const int spl = std::max(P.geom.spl, 1);
-    const int chunk = ((opts->chunk_steps > 0 ? opts->chunk_steps : 64) + spl - 1) / spl * spl;
+    const int chunk = opts->chunk_steps > 0 ? (opts->chunk_steps + spl - 1) / spl * spl
+                                            : default_chunk(P.geom.max_steps - opts->start_step, spl);
     BatchBuffers B = carve(P, workspace_dev);
     char* ws = static_cast<char*>(workspace_dev);
     cudaError_t e;

@@ -120,8 +120,8 @@ struct BatchGeometry {
     int32_t strip_t, strip_g;  // three-step strips: samples side by side and warps per group (StripPacker)
     int32_t strip_closed;    // three-step strips: whole rows fit a warp, lanes wrap around
     int32_t strip_ny;        // three-step strips: the samples' common height (0: heights differ)
-    int32_t pad_;            // keeps the struct free of padding bytes (it keys the graph cache)
 };
+static_assert(sizeof(BatchGeometry) == 3 * 8 + 24 * 4, "no padding bytes: the struct keys the graph cache");
 
 // Output pointers of a run (rows indexed by SampleDev::sample_id).
 struct RunOutputs {
@@ -237,6 +237,7 @@ constexpr int kStripGroupWarps = 64;    // most warps per group
 constexpr int kStripGroupSamples = 6;   // most samples side by side (rows that do not close)
 struct StripMap {
     int32_t samples, warps, closed, nx, ny;  // ny: common height (0: heights differ)
+    int32_t part;  // rows of one group of samples per range (0: equal ranges over all rows)
     uint8_t start[kStripGroupWarps + 4];
     StripStretch stretch[kStripGroupWarps + kStripGroupSamples];
 };
