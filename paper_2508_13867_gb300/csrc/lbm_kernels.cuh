@@ -2622,23 +2622,25 @@ const StripBlocks& strip_regs_blocks() {
 }
 
 // Rows per range of a launch that splits every group of samples into equal parts, 0 where equal ranges
-// over all rows are better (or heights differ).  The time of a launch in units of one phase of one warp: a
-// range of n rows takes n + 2 (NS - 1) iterations one after the other, about five units each, or the
-// work of the busiest SM, NS n + NS (NS - 1) phases of each of its blocks.  Equal ranges take the pieces of
-// two groups where they cross (2 NS (NS - 1) and 4 (NS - 1) instead).  grid: most blocks at once.
+// over all rows are better (or heights differ).  The time of a launch in units of one phase of one block
+// on its SM (0.105 us FP32): a range of n rows takes n full iterations of about eight units each, whatever
+// else runs on the SM (FX16 at two blocks per SM 7.9, FP32 at most 8), and 2 (NS - 1) first ones of half
+// the phases; or the busiest SM takes NS n + NS (NS - 1) phases of each of its blocks.  Equal ranges take
+// the first iterations twice where they cross from one group into the next.  On ties more parts (more
+// warps to hide latency).  grid: most blocks at once.
 inline int strip_part(int64_t nsup, int ny, int warps, int ns, int64_t grid) {
     if (ny <= 0 || nsup * warps > grid * kStripWarps) return 0;
     const int64_t sms = sm_count(), groups = grid * kStripWarps / warps;
     auto cost = [&](int64_t blocks, int64_t n, int64_t pieces) {
-        return std::max(5 * (n + pieces * 2 * (ns - 1)), (blocks + sms - 1) / sms * (ns * n + pieces * ns * (ns - 1)));
+        return std::max(8 * n + pieces * 9 * (ns - 1), (blocks + sms - 1) / sms * (ns * n + pieces * ns * (ns - 1)));
     };
     const int64_t per = (nsup * ny + groups - 1) / groups;
-    int64_t best = cost(grid, per, per >= ny || ny % per != 0 ? 2 : 1);
+    int64_t best = cost(grid, per, per >= ny || ny % per != 0 ? 2 : 1) + 1;
     int part = 0;
     for (int64_t parts = std::min<int64_t>(groups / nsup, ny); parts >= 1; --parts) {
         const int64_t n = (ny + parts - 1) / parts, used = (ny + n - 1) / n;
         const int64_t c = cost((nsup * used * warps + kStripWarps - 1) / kStripWarps, n, 1);
-        if (c <= best) {
+        if (c < best) {
             best = c;
             part = (int)n;
         }
