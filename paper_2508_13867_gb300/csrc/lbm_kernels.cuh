@@ -226,27 +226,47 @@ __device__ __forceinline__ typename Storage<S>::C read_incoming(
     }
 }
 
-// Block-wide deterministic sum of NV doubles; result valid in thread 0.
+// Block-wide deterministic sum of NV doubles; result valid in thread 0.  An FP64 add of a warp holds the
+// SM's FP64 units for 19 cycles, so the values are summed together: at each of the first levels a lane
+// keeps half of the values and sends the other half (7 values: 9 adds per warp instead of 35), and the
+// warps' sums are added by one lane per value.  The pairs and their order are those of one butterfly per
+// value, and so are the bits.
 template <int NV, int NT>
 __device__ __forceinline__ void block_sum(double (&v)[NV], double* smem) {
+    constexpr int P = NV <= 1 ? 1 : (NV <= 2 ? 2 : (NV <= 4 ? 4 : 8));
+    static_assert(NV <= 8, "at most eight values");
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    }
     const int warp = tid >> 5, lane = tid & 31;
-    if (lane == 0) {
+    double a[P];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) smem[warp * NV + k] = v[k];
+    for (int k = 0; k < P; ++k) a[k] = k < NV ? v[k < NV ? k : 0] : 0.0;
+    int at = 0;  // the value this lane ends up with
+#pragma unroll
+    for (int o = 16, m = P / 2; o > 0; o >>= 1, m >>= 1) {
+        if (m > 0) {
+            const bool upper = (lane & o) != 0;
+            at += upper ? m : 0;
+#pragma unroll
+            for (int i = 0; i < m; ++i) {
+                const double keep = upper ? a[i + m] : a[i], send = upper ? a[i] : a[i + m];
+                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        } else {
+            a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+        }
     }
+    if ((lane & (32 / P - 1)) == 0 && at < NV) smem[warp * NV + at] = a[0];
     __syncthreads();
-    if (tid == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
+    if (warp == 0) {
+        if (lane < NV) {
             double s = 0.0;
-            for (int w = 0; w < NT / 32; ++w) s += smem[w * NV + k];
-            v[k] = s;
+            for (int w = 0; w < NT / 32; ++w) s += smem[w * NV + lane];
+            smem[lane] = s;  // only this lane reads or writes its column
+        }
+        __syncwarp();
+        if (lane == 0) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) v[k] = smem[k];
         }
     }
     __syncthreads();
@@ -2031,7 +2051,9 @@ int cluster_capacity(int csize, size_t smem) {
 
 
 // ------------------------------------------------------------------------------------------
-// Final fields and per-sample scalars at the last step run.
+// Final fields and per-sample scalars at the last step run.  Bound by its FP64 instructions (conversions,
+// sums and their reduction; 0.27 ms of HBM at 625 x 256^2 FP32): status in the compute type, sums reduced
+// together (block_sum); 2.1 -> 1.3 ms there, 1.3 -> 0.8 ms at 96 x 512^2.
 // ------------------------------------------------------------------------------------------
 template <typename S, bool MIXED>
 __global__ void __launch_bounds__(256) finalize_kernel(KParams p, int64_t total_tiles, int tile_rows, int tile_cols) {
@@ -2055,6 +2077,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(KParams p, int64_t total_
         S* lat = arena;
         if (two && on_final_second(p, sp.slot, T)) lat = static_cast<S*>(p.arena2);
         double red[7] = {0, 0, 0, 0, 0, 0, 0};  // K, mass, mx, my, fx, fy, bad
+        int bad = 0;
         for (int q = threadIdx.x; q < tile_rows * tile_cols; q += blockDim.x) {
             const int x = (lt % sp.tiles_x) * tile_cols + (q % tile_cols);
             const int y = y0 + q / tile_cols;
@@ -2069,7 +2092,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(KParams p, int64_t total_
                     // a value held at the end of the fixed-point range saturated on a store
 #pragma unroll
                     for (int i = 0; i < 9; ++i)
-                        if (Storage<S>::at_limit(base + i * sp.plane + own)) red[6] += 1.0;
+                        bad += Storage<S>::at_limit(base + i * sp.plane + own) ? 1 : 0;
                 }
                 if (two || p.natural || (T & 1) == 0) {
 #pragma unroll
@@ -2107,7 +2130,8 @@ __global__ void __launch_bounds__(256) finalize_kernel(KParams p, int64_t total_
                 red[1] += rho;
                 red[2] += rho * ux;
                 red[3] += rho * uy;
-                if (!(rho > 0.0) || !isfinite(ux) || !isfinite(uy)) red[6] += 1.0;
+                // rho = 1 + drho > 0
+                if (!(drho > C(-1)) || !isfinite(cux) || !isfinite(cuy)) ++bad;
                 if (mask != nullptr && T > 0) {
                     // halfway: the bounce-back populations at T are the post-collision values of
                     // step T - 1; Bouzidi: c_i (g*_i(T - 1) parked in the obstacle node + the
@@ -2148,6 +2172,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(KParams p, int64_t total_
                 }
             }
         }
+        red[6] = (double)bad;
         double tot[7];
         if (tile_reduce_last<7, NT>(p, sp, j, (int)tile, red, tot, s_red, &s_flag)) {
             if (threadIdx.x == 0) {

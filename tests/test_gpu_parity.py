@@ -1399,3 +1399,20 @@ def test_projection_contractions(dtype, dim, order, pts, quad, F):
         if F > 1:
             assert np.isnan(got[:, F - 1]).all()
     e.close()
+
+
+@pytest.mark.parametrize("n", [5, 31, 40, 129])
+@pytest.mark.parametrize("rows,npt", [(4, 1), (8, 1), (4, 2)])
+def test_sums_over_tiles(ens, n, rows, npt):
+    """The blocks' sums (K in the step kernel; K, mass, momentum and status at the end) over tiles with few
+    and many rows and warps, on lattices that leave lanes and rows of a tile empty, against the oracle: sums
+    of at most 129^2 FP64 terms (the bounds of the FP64 invariants above)."""
+    specs = _tgv_specs(n, 12)
+    g = _run(ens, specs, "f64", qoi_every=3, series=True, tile_rows=rows, npt=npt, scheme="one_step")
+    for i, r in enumerate(olbm.run([oracle_case(s, qoi_every=3) for s in specs])):
+        q = g["qoi"][i]
+        assert abs(q[U.UQLB_QOI_K] - r.k_final) < 1e-12 * abs(r.k_final)
+        assert abs(q[U.UQLB_QOI_MASS] - r.mass) < 1e-12 * r.mass
+        assert max(abs(q[U.UQLB_QOI_MOMX] - r.mom_x), abs(q[U.UQLB_QOI_MOMY] - r.mom_y)) < 1e-12 * r.mass
+        assert q[U.UQLB_QOI_STATUS] == 0
+        assert np.allclose(g["series"][i, :5], r.series[:5], rtol=1e-12, atol=0)
