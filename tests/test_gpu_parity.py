@@ -1416,3 +1416,51 @@ def test_sums_over_tiles(ens, n, rows, npt):
         assert max(abs(q[U.UQLB_QOI_MOMX] - r.mom_x), abs(q[U.UQLB_QOI_MOMY] - r.mom_y)) < 1e-12 * r.mass
         assert q[U.UQLB_QOI_STATUS] == 0
         assert np.allclose(g["series"][i, :5], r.series[:5], rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("storage,nx,ny,every,steps", [
+    ("f32", 256, 256, 9, (10, 9, 9)), ("f32", 256, 256, 3, (104, 101, 101)), ("f32", 66, 8, 5, (12, 10, 9)),
+    ("f32", 127, 127, 7, (22, 21, 20)), ("f32", 57, 6, 2, (7, 6, 5, 4, 3, 2, 1)), ("f32", 48, 5, 3, (4, 3, 3, 2)),
+    ("bf16", 128, 40, 7, (8, 7, 7)), ("fx16", 256, 24, 7, (8, 7, 7)), ("f16", 113, 9, 4, (6, 5, 4, 4, 3))])
+def test_register_strips_of_samples_that_end_around_a_recorded_step(ens, storage, nx, ny, every, steps):
+    """Samples side by side in one group of the three-step strips that end on both sides of a recorded step
+    within one launch: the kinetic energy series, the final QoI row and the K column of every sample, and
+    those of a run resumed on the same workspace, against runs of each sample alone.  The fields are those
+    bits (16-bit storage rounds to nearest, without the sample's random bits); the sums are of the same
+    nx ny terms in another order, each addition off by at most 2^-53 of sums below the mass."""
+    specs = [replace(W.tgv(nx, k, nu=0.03 + 0.01 * (i % 3), u0=0.01), ny=ny) for i, k in enumerate(steps)]
+    first = max(steps)
+    longer = [replace(s, steps=first + 2 * every) if s.steps == first else s for s in specs]
+
+    def run(batch, start=0):
+        out = {"qoi": torch.full((len(batch), U.UQLB_QOI_COLS), -7.0, dtype=torch.float64, device="cuda"),
+               "fields": torch.full((len(batch), 2 * nx * ny + 1), -7.0, dtype=torch.float64, device="cuda")}
+        res = ens.run_batch([sample_struct(s) for s in batch], storage=storage, fields_dtype="f64", qoi_every=every,
+                            series=True, rounding="nearest", scheme="three_step_strips", start_step=start, out=out)
+        torch.cuda.synchronize()
+        return {k: v.cpu().numpy() for k, v in res.items()}
+
+    def check(got, batch, since=0):
+        eps = nx * ny * 2.0 ** -53
+        for i, s in enumerate(batch):
+            one = run([s])
+            assert np.array_equal(got["fields"][i, :-1], one["fields"][0, :-1]), i
+            assert abs(got["fields"][i, -1] - one["fields"][0, -1]) <= 2 * eps * one["fields"][0, -1], i
+            q, r = got["qoi"][i], one["qoi"][0]
+            assert q[U.UQLB_QOI_STEPS] == s.steps and q[U.UQLB_QOI_STATUS] == 0, i
+            assert abs(q[U.UQLB_QOI_K] - r[U.UQLB_QOI_K]) <= 2 * eps * r[U.UQLB_QOI_K], i
+            for c in (U.UQLB_QOI_MASS, U.UQLB_QOI_MOMX, U.UQLB_QOI_MOMY):
+                assert abs(q[c] - r[c]) <= 2 * eps * r[U.UQLB_QOI_MASS], (i, c)
+            at = [k for k in range(s.steps // every + 1) if k * every >= since]
+            assert np.allclose(got["series"][i, at], one["series"][0, at], rtol=2 * eps, atol=0), i
+
+    whole = run(specs)
+    check(whole, specs)
+    assert np.array_equal(run(specs)["qoi"], whole["qoi"])  # the head of the run that is resumed
+    if storage == "f32":  # 16-bit storage rounds once per launch, whose ends a resumed run moves
+        resumed = run(longer, first)
+        for i, s in enumerate(specs):
+            if s.steps < first:
+                assert np.array_equal(resumed["qoi"][i], whole["qoi"][i]), i
+        keep = [i for i, s in enumerate(specs) if s.steps == first]
+        check({k: v[keep] for k, v in resumed.items()}, [longer[i] for i in keep], first)
