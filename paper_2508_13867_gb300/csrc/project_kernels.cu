@@ -460,8 +460,10 @@ template <typename M>
 cudaError_t launch_refl(const ReflPlanView& p, int K, const M* m, int64_t F, int64_t ld, double* C, cudaStream_t s) {
     const int hrows = 1 << p.max_m;
     const size_t smem = (size_t)(K + hrows) * kReflThreads * sizeof(double);
-    static const cudaError_t opt_in = cudaFuncSetAttribute(reflect_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           kReflMaxRows * kReflThreads * (int)sizeof(double));
+    // the limit belongs to the current device, so it is set for each launch; always the same value, as
+    // threads of one process may launch at once
+    const cudaError_t opt_in = cudaFuncSetAttribute(reflect_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    kReflMaxRows * kReflThreads * (int)sizeof(double));
     if (opt_in != cudaSuccess) return opt_in;
     reflect_kernel<M><<<(unsigned)((F + kReflThreads - 1) / kReflThreads), kReflThreads, smem, s>>>(
         p.orbits, p.norbits, p.terms, p.members, K, hrows, m, F, ld, C);
