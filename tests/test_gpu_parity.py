@@ -1464,3 +1464,51 @@ def test_register_strips_of_samples_that_end_around_a_recorded_step(ens, storage
                 assert np.array_equal(resumed["qoi"][i], whole["qoi"][i]), i
         keep = [i for i, s in enumerate(specs) if s.steps == first]
         check({k: v[keep] for k, v in resumed.items()}, [longer[i] for i in keep], first)
+
+
+def _device_us(fn):
+    """Shortest device time of ten calls in microseconds."""
+    fn()
+    best = math.inf
+    for _ in range(10):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        fn()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, 1e3 * a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("rows,nodes,bins", [(3, 1, 1), (700, 4, 64), (5000, 3, 8192), (257, 225, 4096), (2, 40000, 8192),
+                                             (900, 255, 8193), (11, 2049, 1 << 20)])
+def test_w1_is_exact_for_rows_of_any_length(ens, dtype, rows, nodes, bins):
+    """The distance against sum |n_b C_a - n_a C_b| in Python integers (C: cumulative counts), which the kernel
+    forms exactly: five roundings (sum, product of the counts, quotient, bin width, product) of 2^-53.  The
+    values are FP32 numbers, so that squares are exact in FP64 and no speed is near an edge by rounding."""
+    rng = np.random.default_rng(rows + bins)
+    sets = [(0.01 * (1 + 0.2 * k) * rng.standard_normal((r, 2 * nodes + 1))).astype(np.float32)
+            for k, r in enumerate((rows, max(1, rows // 2)))]
+    w1, bound, bad = ens.w1_speed(*(x for m in sets for x in (torch.from_numpy(m.astype(dtype)).cuda(), nodes)), bins=bins)
+    sp = [np.sqrt(m[:, :nodes].astype(np.float64) ** 2 + m[:, nodes: 2 * nodes].astype(np.float64) ** 2).ravel()
+          for m in sets]
+    vmax = max(s.max() for s in sp)
+    na, nb = len(sp[0]), len(sp[1])
+    ca, cb = (np.cumsum(np.bincount(np.minimum((s * (bins / vmax)).astype(np.int64), bins - 1), minlength=bins))
+              for s in sp)
+    exact = sum(abs(int(x) * nb - int(y) * na) for x, y in zip(ca, cb)) / (na * nb) * (vmax / bins)
+    assert bound == vmax / bins and tuple(bad) == (0, 0)
+    assert abs(w1 - exact) <= 8 * 2.0 ** -53 * exact
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_w1_takes_no_longer_for_short_rows(ens, dtype):
+    """One million speeds in rows of four nodes and in one row: the same work, so well within a factor of
+    three of each other (a kernel that takes one row at a time needs ten times as long and more)."""
+    m = 0.01 * torch.randn((250000, 9), device="cuda", dtype=dtype)
+    one = torch.cat([m[:, :4].reshape(1, -1), m[:, 4:8].reshape(1, -1), m[:1, :1]], dim=1).contiguous()
+    got = [ens.w1_speed(x, n, x, n, bins=1 << 16)[1] for x, n in ((m, 4), (one, 1000000))]
+    assert got[0] == got[1]
+    short = _device_us(lambda: ens.w1_speed(m, 4, m, 4, bins=1 << 16))
+    assert short < 3 * _device_us(lambda: ens.w1_speed(one, 1000000, one, 1000000, bins=1 << 16))
