@@ -1512,3 +1512,13 @@ def test_w1_takes_no_longer_for_short_rows(ens, dtype):
     assert got[0] == got[1]
     short = _device_us(lambda: ens.w1_speed(m, 4, m, 4, bins=1 << 16))
     assert short < 3 * _device_us(lambda: ens.w1_speed(one, 1000000, one, 1000000, bins=1 << 16))
+
+
+@pytest.mark.parametrize("dtype,bins,n", [(torch.float32, 8192, 250000), (torch.float64, 8192, 250000),
+                                          (torch.float64, 4096, 65536), (torch.float32, 1, 2000)])
+def test_w1_takes_no_longer_for_few_bins(ens, dtype, bins, n):
+    """Few bins are counted in shared memory: no slower than 65536 bins in global memory (which also scan
+    eight times as many bins) by more than a half.  Too few blocks took three to six times as long."""
+    m = 0.01 * torch.randn((1, 2 * n + 1), device="cuda", dtype=dtype)
+    few = _device_us(lambda: ens.w1_speed(m, n, m, n, bins=bins))
+    assert few < 1.5 * _device_us(lambda: ens.w1_speed(m, n, m, n, bins=1 << 16))
