@@ -3,8 +3,9 @@
 //   coefficients (Eq. coef_discrete, gamma_k = 1):  C[k, f] = sum_s W[k, s] M[s, f],
 //                                                     W[k, s] = a_s Phi_k(xi_s)
 //   gPC mean / variance (Eq. gpc_mean, Eq. gpc_std):  mean = C[0, f], var = sum_{k>=1} C[k, f]^2
-//   Monte Carlo (Eq. meanMCS, Eq. varMCS):           two passes over the samples
-// All accumulation is FP64; M may be FP32 (the ensemble's field output) or FP64.
+//   Monte Carlo (Eq. meanMCS, Eq. varMCS):           two passes over the samples in FP64, or (FP32 fields of
+//     many samples) one pass with sums of three FP32 numbers
+// All other accumulation is FP64; M may be FP32 (the ensemble's field output) or FP64.
 // The contraction is [K x S] x [S x F] with K <= a few hundred and F up to ~10^6.  Three forms: one input at
 // a time on tensor grids (sf_stage_kernel), over reflected samples on symmetric sample sets
 // (reflect_kernel), dense (project_kernel).
@@ -190,7 +191,7 @@ __global__ void mc_stats_kernel(const M* __restrict__ m, int64_t S, int64_t F, i
 // cancellation of the shift costs nothing.  A field with a non-finite value, or a deviation outside
 // [1e-15, 1e15] (whose square or its rounding error would leave FP32's range), is left to FP64.
 // A block takes 32 fields, each of its eight warps every eighth sample.  Measured on 1024 samples of 2 x
-// 512^2 + 1 fields: 0.92 against 5.09 ms.
+// 512^2 + 1 fields: 0.92 against 5.09 ms (mc_one_pass() says for which sizes).
 constexpr int kMcWarps = 8;
 struct Sum3 {
     float a, b, c;
@@ -513,6 +514,16 @@ cudaError_t launch_gpc_stats(const double* C, int K, int64_t F, double* mean, do
     return cudaGetLastError();
 }
 
+// FP32 fields: one pass or two.  The merge of the warps' sums and the pairs of one pass cost some 60 FP64
+// instructions per field whatever S is, the two passes five per value, so few samples of many fields take
+// two; few fields do not fill the chip, and there the chains of the two passes are the longer ones.  One
+// pass / two passes in us: 131073 fields 4 samples 45 / 28, 12 47 / 39, 16 48 / 46, 20 49 / 52; 524289 fields
+// 4 123 / 55, 16 134 / 116, 20 141 / 136, 24 142 / 156; 2097153 fields 12 541 / 319, 24 600 / 548, 32 649 / 702;
+// 32769 fields 4 27 / 24, 12 28 / 25, 20 28 / 28; 16385 fields 4 21 / 23, 16 22 / 25.
+static bool mc_one_pass(int64_t S, int64_t F) {
+    return F < (1 << 15) || S >= (F < (1 << 18) ? 16 : (F < (1 << 20) ? 20 : 28));
+}
+
 cudaError_t launch_mc_stats(const void* M, int dtype, int64_t S, int64_t F, int64_t ld, double* mean,
                             double* var, int ddof, cudaStream_t s) {
     if (F <= 0) return cudaSuccess;
@@ -520,6 +531,8 @@ cudaError_t launch_mc_stats(const void* M, int dtype, int64_t S, int64_t F, int6
     const unsigned g = (unsigned)(blocks < 65535 * 8 ? blocks : 65535 * 8);
     if (dtype == UQLB_F64)
         mc_stats_kernel<double><<<g, 256, 0, s>>>(static_cast<const double*>(M), S, F, ld, mean, var, ddof);
+    else if (!mc_one_pass(S, F))
+        mc_stats_kernel<float><<<g, 256, 0, s>>>(static_cast<const float*>(M), S, F, ld, mean, var, ddof);
     else
         mc_stats_f32_kernel<<<(unsigned)((F + 31) / 32), dim3(32, kMcWarps), 0, s>>>(static_cast<const float*>(M), S, F, ld,
                                                                                      mean, var, ddof);

@@ -1522,3 +1522,37 @@ def test_w1_takes_no_longer_for_few_bins(ens, dtype, bins, n):
     m = 0.01 * torch.randn((1, 2 * n + 1), device="cuda", dtype=dtype)
     few = _device_us(lambda: ens.w1_speed(m, n, m, n, bins=bins))
     assert few < 1.5 * _device_us(lambda: ens.w1_speed(m, n, m, n, bins=1 << 16))
+
+
+@pytest.mark.parametrize("S,F", [(15, 32767), (15, 32768), (16, 32768), (19, 262144), (20, 262144), (27, 1048576),
+                                 (28, 1048576)])
+def test_mc_statistics_on_both_sides_of_one_pass(S, F):
+    """FP32 fields where the kernel changes from two passes to one, against FP64 on the device: S rounding
+    errors of 2^-53 for the mean (of values within 2 of each other's size), S + 4 for the variance, twice
+    (both sides round)."""
+    e = Ensemble(0)
+    e.set_inputs([(0.0, 1.0)])
+    e.init_mc(S, 1)
+    m = 1.0 + 0.1 * torch.rand((S, F), device="cuda")
+    mean, var = e.stats(m)
+    x = m.double()
+    mu = x.mean(0)
+    ref = ((x - mu) ** 2).sum(0) / (S - 1)
+    assert float(((mean - mu).abs() / mu).max()) <= 2 * S * 2.0 ** -53
+    assert float(((var - ref).abs() / ref).max()) <= 2 * (S + 4) * 2.0 ** -53
+    e.close()
+
+
+@pytest.mark.parametrize("S", [2, 4, 8, 15, 16])
+def test_mc_statistics_of_few_fp32_samples_take_no_longer_than_fp64(S):
+    """Mean and variance of a few samples of many fields: half the bytes of FP64 fields and one conversion
+    more per value, so within a factor of two of them (the sums of three FP32 numbers, which pay for many
+    samples, took up to 3.5 times as long for few)."""
+    F = 1 << 21
+    e = Ensemble(0)
+    e.set_inputs([(0.0, 1.0)])
+    e.init_mc(S, 1)
+    m = torch.randn((S, F), device="cuda")
+    m64 = m.double()
+    assert _device_us(lambda: e.stats(m)) < 2 * _device_us(lambda: e.stats(m64))
+    e.close()
