@@ -353,7 +353,48 @@ __device__ __forceinline__ void sf_group(const TI* src, int64_t step, const doub
     for (int a = 0; a < CNT; ++a) out[(int64_t)__ldg(o + a) * out_ld] = y[a];
 }
 
-// N: points per input (0: runtime n, the degrees one after the other).
+// The same for n points that are not compiled in, without the fold: the inputs are loaded and converted once,
+// and the degrees are CNT independent chains, eight inputs in flight (four lose 11 % at five degrees and 10
+// points, gain 7 % at two).  Measured with the statistics, FP32 / FP64 fields, 131073 fields: 16 x 16 points at
+// degree 8 756 / 678 us, 10 x 10 at degree 4 195 / 167; one degree after the other, which reloads and
+// converts the inputs for each, 1288 / 681 and 296 / 168; all nine degrees with predicates 887 / 813, 357 / 329.
+template <int CNT, typename TI>
+__device__ __forceinline__ void sf_group_any(const TI* src, int64_t step, int n, const double (*G)[kSfMaxPoints],
+                                             double* out, int64_t out_ld, const int* __restrict__ o) {
+    double y[CNT];
+#pragma unroll
+    for (int a = 0; a < CNT; ++a) y[a] = 0.0;
+#pragma unroll (CNT <= 2 ? 4 : 8)
+    for (int q = 0; q < n; ++q) {
+        const double x = (double)src[q * step];
+#pragma unroll
+        for (int a = 0; a < CNT; ++a) y[a] = fma(G[a][q], x, y[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < CNT; ++a) out[(int64_t)__ldg(o + a) * out_ld] = y[a];
+}
+
+// Calls an expression with the compile-time count C of admitted degrees.
+#define UQLB_SF_CASE(C_, CALL) \
+    case C_: { \
+        constexpr int C = C_; \
+        CALL; \
+        break; \
+    }
+#define UQLB_SF_SWITCH(...) \
+    switch (cnt) { \
+        UQLB_SF_CASE(1, (__VA_ARGS__)) \
+        UQLB_SF_CASE(2, (__VA_ARGS__)) \
+        UQLB_SF_CASE(3, (__VA_ARGS__)) \
+        UQLB_SF_CASE(4, (__VA_ARGS__)) \
+        UQLB_SF_CASE(5, (__VA_ARGS__)) \
+        UQLB_SF_CASE(6, (__VA_ARGS__)) \
+        UQLB_SF_CASE(7, (__VA_ARGS__)) \
+        UQLB_SF_CASE(8, (__VA_ARGS__)) \
+        UQLB_SF_CASE(9, (__VA_ARGS__)) \
+    }
+
+// N: points per input (0: runtime n).
 template <typename TI, int N>
 __global__ void __launch_bounds__(kSfThreads) sf_stage_kernel(const TI* __restrict__ in, int64_t in_ld,
                                                               double* __restrict__ out, int64_t out_ld,
@@ -384,26 +425,9 @@ __global__ void __launch_bounds__(kSfThreads) sf_stage_kernel(const TI* __restri
         const int64_t step = (int64_t)jprev * in_ld;
         double* dst = out + (r * jout) * out_ld + f;
         if constexpr (N > 0) {
-            switch (cnt) {
-#define UQLB_SF_CASE(C_) \
-    case C_: sf_group<N, C_>(src, step, sG, dst, out_ld, o); break;
-                UQLB_SF_CASE(1)
-                UQLB_SF_CASE(2)
-                UQLB_SF_CASE(3)
-                UQLB_SF_CASE(4)
-                UQLB_SF_CASE(5)
-                UQLB_SF_CASE(6)
-                UQLB_SF_CASE(7)
-                UQLB_SF_CASE(8)
-                UQLB_SF_CASE(9)
-#undef UQLB_SF_CASE
-            }
+            UQLB_SF_SWITCH(sf_group<N, C>(src, step, sG, dst, out_ld, o))
         } else {
-            for (int a = 0; a < cnt; ++a) {
-                double y = 0.0;
-                for (int q = 0; q < n; ++q) y = fma(sG[a][q], (double)src[q * step], y);
-                dst[(int64_t)__ldg(o + a) * out_ld] = y;
-            }
+            UQLB_SF_SWITCH(sf_group_any<C>(src, step, n, sG, dst, out_ld, o))
         }
     }
 }

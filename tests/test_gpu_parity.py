@@ -1556,3 +1556,20 @@ def test_mc_statistics_of_few_fp32_samples_take_no_longer_than_fp64(S):
     m64 = m.double()
     assert _device_us(lambda: e.stats(m)) < 2 * _device_us(lambda: e.stats(m64))
     e.close()
+
+
+@pytest.mark.parametrize("dim,order,pts", [(2, 8, 16), (1, 8, 12), (2, 5, 10), (2, 0, 11)])
+def test_projection_of_many_points_converts_its_inputs_once(dim, order, pts):
+    """Tensor grids of more points per input than are compiled in, FP32 fields: half the bytes of FP64 fields and
+    one conversion per value, so at most about (degrees + 1) / degrees of their time where the FP64 units bound
+    both (up to a half more with loads); a conversion for each degree took 1.8 times as long.  Equal bits."""
+    e = Ensemble(0)
+    e.set_inputs([(-1.0, 1.0)] * dim)
+    e.init_gpc(order, pts)
+    m = torch.randn((e.num_samples, 131072), device="cuda")
+    m64 = m.double()
+    c = torch.empty((e.num_terms, m.shape[1]), dtype=torch.float64, device="cuda")
+    c64 = torch.empty_like(c)
+    assert _device_us(lambda: e.project(m, c)) < 1.5 * _device_us(lambda: e.project(m64, c64))
+    assert torch.equal(c, c64)
+    e.close()
