@@ -9,6 +9,7 @@
 // The contraction is [K x S] x [S x F] with K <= a few hundred and F up to ~10^6.  Three forms: one input at
 // a time on tensor grids (sf_stage_kernel), over reflected samples on symmetric sample sets
 // (reflect_kernel), dense (project_kernel).
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <mutex>
@@ -25,9 +26,9 @@ constexpr int kSB = 128;  // samples per shared-memory stage
 
 // Dense contraction, KB coefficients per block (blockIdx.y chunk) and FPT fields per thread.  FP64
 // instructions bound it (one per warp in 19 cycles of an SM), so a term block that divides K badly costs
-// in proportion: launch_project takes the KB with the least work for K (K = 35: 37 instructions
+// in proportion: launch_dense_any() takes the KB with the least work for K (K = 35: 37 instructions
 // per sample in one block of 36 against 51 in three of 16; the conversion of a value is shared by the
-// block's terms).
+// block's terms), or the smallest blocks where few fields leave SMs idle.
 template <typename M, int KB, int FPT>
 __global__ void __launch_bounds__(kProjThreads) project_kernel(const double* __restrict__ W, int K, int S,
                                                                const M* __restrict__ m, int64_t F, int64_t ld,
@@ -462,13 +463,21 @@ void launch_dense(const double* W, int K, int S, const M* m, int64_t F, int64_t 
 }
 template <typename M>
 void launch_dense_any(const double* W, int K, int S, const M* m, int64_t F, int64_t ld, double* C, cudaStream_t s) {
-    // FP64 instructions per field and sample of a block size: its terms and one conversion, per block
-    constexpr int kSizes[] = {6, 12, 16, 24, 36};
-    int best = 0, cost = 0;
-    for (int kb : kSizes) {
-        const int c = (K + kb - 1) / kb * (kb + 1);
+    // FP64 instructions per sample of the busiest SM: a thread's terms and conversions times the blocks per SM.
+    // One block saturates its SM's FP64 units, so many fields go by the total work alone, and few, which
+    // leave SMs idle, take small blocks (137 samples, 70 terms, 2049 fields: 98 us, by total work 222; 41 samples,
+    // 35 terms, 129 fields 39 / 79).
+    struct Size {
+        int kb, fpt;
+    };
+    constexpr Size kSizes[] = {{6, 2}, {12, 2}, {16, 2}, {24, 1}, {36, 1}};
+    int best = 0;
+    double cost = 0.0;
+    for (const Size& z : kSizes) {
+        const int64_t blocks = (F + kProjThreads * z.fpt - 1) / (kProjThreads * z.fpt) * ((K + z.kb - 1) / z.kb);
+        const double c = std::max(blocks / 152.0, 1.0) * (z.fpt * (z.kb + 1));
         if (best == 0 || c < cost) {
-            best = kb;
+            best = z.kb;
             cost = c;
         }
     }
@@ -485,11 +494,13 @@ template <typename M>
 cudaError_t launch_refl(const ReflPlanView& p, int K, const M* m, int64_t F, int64_t ld, double* C, cudaStream_t s) {
     const int hrows = 1 << p.max_m;
     const size_t smem = (size_t)(K + hrows) * kReflThreads * sizeof(double);
-    // the limit belongs to the current device, so it is set for each launch; always the same value, as
-    // threads of one process may launch at once
-    const cudaError_t opt_in = cudaFuncSetAttribute(reflect_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                    kReflMaxRows * kReflThreads * (int)sizeof(double));
-    if (opt_in != cudaSuccess) return opt_in;
+    if (smem > 48 * 1024) {
+        // the limit belongs to the current device, so it is set for each launch that needs it (1.5 us on the
+        // host); always the same value, as threads of one process may launch at once
+        const cudaError_t e = cudaFuncSetAttribute(reflect_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   kReflMaxRows * kReflThreads * (int)sizeof(double));
+        if (e != cudaSuccess) return e;
+    }
     reflect_kernel<M><<<(unsigned)((F + kReflThreads - 1) / kReflThreads), kReflThreads, smem, s>>>(
         p.orbits, p.norbits, p.terms, p.members, K, hrows, m, F, ld, C);
     return cudaGetLastError();

@@ -1573,3 +1573,18 @@ def test_projection_of_many_points_converts_its_inputs_once(dim, order, pts):
     assert _device_us(lambda: e.project(m, c)) < 1.5 * _device_us(lambda: e.project(m64, c64))
     assert torch.equal(c, c64)
     e.close()
+
+
+def test_dense_projection_of_few_fields_spreads_its_terms(ens):
+    """Few fields leave SMs idle, so 35 terms take little longer than 5 (a block that held all of them took
+    twice as long and more)."""
+    t = []
+    for order in (1, 3):
+        e = Ensemble(0)
+        e.set_inputs([(-1.0, 1.0)] * 4)
+        e.init_gpc(order, 5)
+        m = torch.randn((e.num_samples, 129), device="cuda")
+        c = torch.empty((e.num_terms, 129), dtype=torch.float64, device="cuda")
+        t.append(_device_us(lambda: e.project_block(m, 0, c)))
+        e.close()
+    assert t[1] < 1.5 * t[0]
