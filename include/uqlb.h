@@ -523,7 +523,7 @@ int uqlb_project_workspace_bytes(const uqlb_ctx* ctx, int64_t n_fields, size_t* 
  *   over reflected samples, on other sample sets that are symmetric in every input (Clenshaw-Curtis
  *     Smolyak grids) with at most four nonzero reference coordinates per sample and K up to about 100, in a
  *     16-byte aligned workspace of uqlb_post_workspace_bytes: samples that differ in signs only are summed
- *     with their signs first;
+ *     with their signs first (few fields of many terms per sample: dense, which is the shorter chain then);
  *   dense, [K x S] x [S x n_fields], with a workspace below the first's and for every other sample set
  *     (uqlb_post_workspace_bytes).
  * uqlb_last_projection reports which one the last call took. */

@@ -535,6 +535,15 @@ cudaError_t launch_project(const double* W, int K, int S, const void* M, int dty
     return cudaGetLastError();
 }
 
+// Over reflected samples or dense.  Few fields leave SMs idle under either, and a call is then a chain: 0.70 us
+// per orbit and 0.086 per term (its sum lies in shared memory) against 0.56 per sample for blocks of six
+// terms (fit of 14 sparse grids, one field, to 3 us).  On many terms per sample the dense chain is the shorter
+// one: 69 samples x 84 terms, 129 fields 114 us over reflected samples, 56 dense; 177 x 35 156, 113.
+bool reflect_pays(int K, int64_t S, int64_t F, int norbits, int nterms) {
+    const int64_t blocks = (F + 2 * kProjThreads - 1) / (2 * kProjThreads) * ((K + 5) / 6);
+    return blocks > 152 || 0.70 * norbits + 0.086 * nterms <= 0.56 * (double)S;
+}
+
 cudaError_t launch_reflect(const ReflPlanView& p, int K, const void* M, int dtype, int64_t F, int64_t ld, double* C,
                            cudaStream_t s) {
     if (F <= 0 || K <= 0) return cudaSuccess;

@@ -62,7 +62,7 @@ struct uqlb_ctx {
     } sf;
     // Contraction over reflected samples (norbits = 0: not available): orbits, terms and sample indices
     struct ReflPlan {
-        int norbits = 0, max_m = 0;
+        int norbits = 0, nterms = 0, max_m = 0;
         size_t terms_at = 0, members_at = 0;  // byte offsets into tables (orbits first)
         std::vector<unsigned char> tables;
     } refl;
@@ -1540,6 +1540,7 @@ void build_reflection_plan(uqlb_ctx* ctx) {
     std::memcpy(P.tables.data() + P.terms_at, terms.data(), terms.size() * sizeof(ReflTerm));
     std::memcpy(P.tables.data() + P.members_at, members.data(), members.size() * sizeof(int32_t));
     P.max_m = max_m;
+    P.nterms = (int)terms.size();
     P.norbits = (int)ob.size();
 }
 
@@ -2226,7 +2227,8 @@ int uqlb_project(uqlb_ctx* ctx, const void* m_dev, int dtype, int64_t n_fields, 
     size_t need = 0;
     uqlb_post_workspace_bytes(ctx, &need);
     if (workspace_bytes < need) return set_err(ctx, UQLB_ERR_OOM, "project: workspace of %zu bytes, need %zu", workspace_bytes, need);
-    if (ctx->refl.norbits > 0 && reinterpret_cast<uintptr_t>(workspace_dev) % 16 == 0) {
+    if (ctx->refl.norbits > 0 && reinterpret_cast<uintptr_t>(workspace_dev) % 16 == 0 &&
+        reflect_pays(ctx->K, ctx->S, n_fields, ctx->refl.norbits, ctx->refl.nterms)) {
         const auto& P = ctx->refl;
         const char* ws = static_cast<const char*>(workspace_dev);
         e = cudaMemcpyAsync(workspace_dev, P.tables.data(), P.tables.size(), cudaMemcpyHostToDevice, s);

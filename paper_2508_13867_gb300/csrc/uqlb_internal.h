@@ -297,6 +297,7 @@ constexpr int kReflMaxDims = 4;    // nonzero coordinates of a sample
 constexpr int kReflMaxRows = 128;  // K + 2^m rows of per-thread values in shared memory
 cudaError_t launch_reflect(const ReflPlanView& p, int K, const void* M, int dtype, int64_t F, int64_t ld, double* C,
                            cudaStream_t s);
+bool reflect_pays(int K, int64_t S, int64_t F, int norbits, int nterms);
 cudaError_t launch_project(const double* W, int K, int S, const void* M, int dtype,
                            int64_t F, int64_t ld, double* C, cudaStream_t s);
 cudaError_t launch_gpc_stats(const double* C, int K, int64_t F, double* mean, double* var,

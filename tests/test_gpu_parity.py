@@ -1588,3 +1588,22 @@ def test_dense_projection_of_few_fields_spreads_its_terms(ens):
         t.append(_device_us(lambda: e.project_block(m, 0, c)))
         e.close()
     assert t[1] < 1.5 * t[0]
+
+
+def test_sparse_grid_projection_of_few_fields_takes_the_shorter_chain():
+    """69 samples and 84 terms: few fields take the dense contraction (as project_block does, with a
+    synchronisation besides), many the one over reflected samples, with the same coefficients to the rounding
+    of 69 products, 2 x 69 x 2^-53 sum |W| |M|."""
+    e = Ensemble(0)
+    e.set_inputs([(-1.0, 1.0)] * 3)
+    U.uqlb_init_gpc(e.ctx, 6, 3, 0, 1)
+    S, K = e.num_samples, e.num_terms
+    m = torch.randn((S, 40000), device="cuda")
+    few = m[:, :129].contiguous()
+    whole, c = e.project(m), e.project(few)
+    bound = 2 * S * 2.0 ** -53 * np.abs(U.uqlb_get_weight_matrix(e.ctx)) @ np.abs(few.double().cpu().numpy())
+    assert np.all(np.abs((whole[:, :129] - c).cpu().numpy()) <= bound)
+    assert torch.equal(c, e.project_block(few, 0))
+    assert _device_us(lambda: e.project(few, c)) < 1.3 * _device_us(lambda: e.project_block(few, 0, c))
+    assert _device_us(lambda: e.project(m, whole)) < 0.6 * _device_us(lambda: e.project_block(m, 0, whole))
+    e.close()
