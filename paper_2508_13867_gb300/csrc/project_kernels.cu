@@ -9,7 +9,6 @@
 // The contraction is [K x S] x [S x F] with K <= a few hundred and F up to ~10^6.  Three forms: one input at
 // a time on tensor grids (sf_stage_kernel), over reflected samples on symmetric sample sets
 // (reflect_kernel), dense (project_kernel).
-#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <mutex>
@@ -472,10 +471,10 @@ void launch_dense_any(const double* W, int K, int S, const M* m, int64_t F, int6
     };
     constexpr Size kSizes[] = {{6, 2}, {12, 2}, {16, 2}, {24, 1}, {36, 1}};
     int best = 0;
-    double cost = 0.0;
+    int64_t cost = 0;
     for (const Size& z : kSizes) {
         const int64_t blocks = (F + kProjThreads * z.fpt - 1) / (kProjThreads * z.fpt) * ((K + z.kb - 1) / z.kb);
-        const double c = std::max(blocks / 152.0, 1.0) * (z.fpt * (z.kb + 1));
+        const int64_t c = (blocks + 151) / 152 * (z.fpt * (z.kb + 1));
         if (best == 0 || c < cost) {
             best = z.kb;
             cost = c;
