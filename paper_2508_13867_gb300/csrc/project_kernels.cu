@@ -75,15 +75,18 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(const double* __r
     }
 }
 
+// In integers: an FP64 comparison takes the units that bound these kernels.
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
+
 // Contraction over reflected samples.  A sample set that is symmetric in every input (Clenshaw-Curtis
 // Smolyak and Gauss-Legendre grids) falls into orbits of 2^m samples that differ in the signs of their m
 // nonzero reference coordinates.  The weights of a term over an orbit are equal up to the sign that its
 // odd degrees give, so with the signed sums h[p] = sum_b (-1)^(p.b) M[s_b] (m 2^m additions) an orbit adds
 // w_k h[p_k] to term k, and nothing to terms of odd degree in a zero coordinate: 549 multiply-adds and 272
 // additions per field where the dense contraction of 137 samples and 35 terms takes 4795.  Per-thread sums
-// lie in shared memory (a term's index is data).  A field with a non-finite value takes the products one
-// by one, zero weights included, as the dense contraction does.  Measured, 137 samples x 35 terms x 130051
-// fields: 0.36 against 1.66 ms dense (with the statistics).
+// lie in shared memory (a term's index is data).  A field with a non-finite value, or whose signed sums
+// leave the range of FP64, takes the products one by one, zero weights included, as the dense contraction
+// does.  Measured, 137 samples x 35 terms x 130051 fields: 0.36 against 1.66 ms dense (with the statistics).
 constexpr int kReflThreads = 128;
 template <typename M>
 __global__ void __launch_bounds__(kReflThreads) reflect_kernel(const ReflOrbit* __restrict__ orbits, int norbits,
@@ -113,7 +116,7 @@ __global__ void __launch_bounds__(kReflThreads) reflect_kernel(const ReflOrbit* 
                     v[b] = x + y;
                     v[b | 1 << d] = x - y;
                 }
-        finite = finite && isfinite(v[0]);
+        finite = finite && !not_finite(v[0]);
 #pragma unroll
         for (int b = 0; b < N; ++b) hs[b * kReflThreads] = v[b];
         for (int q = o.term; q < o.term + o.nterms; ++q) {
@@ -130,6 +133,11 @@ __global__ void __launch_bounds__(kReflThreads) reflect_kernel(const ReflOrbit* 
             case 3: orbit(std::integral_constant<int, 3>{}, o); break;
             default: orbit(std::integral_constant<int, 4>{}, o); break;
         }
+    }
+    for (int k = 0; k < K; ++k) {
+        const double c = acc[k * kReflThreads];
+        finite = finite && !not_finite(c);  // a difference can leave FP64's range where the sum v[0] does not
+        C[(int64_t)k * F + f] = c;
     }
     if (!finite) {
         for (int k = 0; k < K; ++k) acc[k * kReflThreads] = 0.0;
@@ -148,8 +156,8 @@ __global__ void __launch_bounds__(kReflThreads) reflect_kernel(const ReflOrbit* 
                 }
             }
         }
+        for (int k = 0; k < K; ++k) C[(int64_t)k * F + f] = acc[k * kReflThreads];
     }
-    for (int k = 0; k < K; ++k) C[(int64_t)k * F + f] = acc[k * kReflThreads];
 }
 
 __global__ void gpc_stats_kernel(const double* __restrict__ C, int K, int64_t F, double* mean, double* var) {
@@ -324,13 +332,14 @@ __global__ void __launch_bounds__(32 * kMcWarps) mc_stats_f32_kernel(const float
 // The points of a Gauss-Legendre rule are symmetric, so G[a][n-1-q] = (-1)^a G[a][q] up to rounding: with the
 // sums and differences of opposite inputs a degree takes half the multiply-adds (n = 5, five degrees: 4
 // additions and 15 multiply-adds instead of 25; the middle input keeps its rounding-sized weight in the
-// odd degrees, so that a non-finite value reaches every coefficient).  Points and degrees are compile-time
-// (a runtime bound left the unrolled multiply-adds of 16 points and 9 degrees in the loop, predicated
-// off).  Measured on 625 samples x 131073 fields, all four stages: 1.43 against 3.88 ms (with the statistics).
+// odd degrees, so that a non-finite value reaches every coefficient; a thread with a non-finite result takes
+// the products one by one).  Points and degrees are compile-time (a runtime bound left the unrolled
+// multiply-adds of 16 points and 9 degrees in the loop, predicated off).  Measured on 625 samples x 131073 fields, all four stages: 1.43 against 3.88 ms (with the statistics).
 constexpr int kSfThreads = 256;
 
+// One group of N points; true if its folded inputs left the range of FP64 (or were not finite).
 template <int N, int CNT, typename TI>
-__device__ __forceinline__ void sf_group(const TI* src, int64_t step, const double (*G)[kSfMaxPoints], double* out,
+__device__ __forceinline__ bool sf_group(const TI* src, int64_t step, const double (*G)[kSfMaxPoints], double* out,
                                          int64_t out_ld, const int* __restrict__ o) {
     constexpr int H = N / 2;
     double x[N], e[H > 0 ? H : 1], d[H > 0 ? H : 1];
@@ -351,6 +360,9 @@ __device__ __forceinline__ void sf_group(const TI* src, int64_t step, const doub
     }
 #pragma unroll
     for (int a = 0; a < CNT; ++a) out[(int64_t)__ldg(o + a) * out_ld] = y[a];
+    // a non-finite input, sum or difference of inputs reaches the first even or the first odd degree, whose
+    // weights have no zeros; FP32 inputs have no sums beyond FP64's range
+    return sizeof(TI) == 8 && N > 1 && (not_finite(y[0]) || (CNT > 1 && not_finite(y[CNT > 1 ? 1 : 0])));
 }
 
 // The same for n points that are not compiled in, without the fold: the inputs are loaded and converted once,
@@ -415,6 +427,7 @@ __global__ void __launch_bounds__(kSfThreads) sf_stage_kernel(const TI* __restri
     __syncthreads();
     const int64_t f = (int64_t)blockIdx.x * kSfThreads + threadIdx.x;
     if (f >= F) return;  // no barrier below
+    bool redo = false;
     for (int64_t g = blockIdx.y; g < groups; g += gridDim.y) {
         const int64_t r = g / jprev;
         const int jp = (int)(g - r * jprev);
@@ -425,9 +438,23 @@ __global__ void __launch_bounds__(kSfThreads) sf_stage_kernel(const TI* __restri
         const int64_t step = (int64_t)jprev * in_ld;
         double* dst = out + (r * jout) * out_ld + f;
         if constexpr (N > 0) {
-            UQLB_SF_SWITCH(sf_group<N, C>(src, step, sG, dst, out_ld, o))
+            UQLB_SF_SWITCH(redo |= sf_group<N, C>(src, step, sG, dst, out_ld, o))
         } else {
             UQLB_SF_SWITCH(sf_group_any<C>(src, step, n, sG, dst, out_ld, o))
+        }
+    }
+    if (!redo) return;
+    // this thread's groups once more, product by product (after the loop: tests and a second path within it
+    // cost the 625 samples x 131073 fields 6 %)
+    for (int64_t g = blockIdx.y; g < groups; g += gridDim.y) {
+        const int64_t r = g / jprev;
+        const int jp = (int)(g - r * jprev);
+        for (int a = 0; a < p1; ++a) {
+            const int to = __ldg(oidx + jp * p1 + a);
+            if (to < 0) break;
+            double y = 0.0;
+            for (int q = 0; q < n; ++q) y = fma(sG[a][q], (double)in[((r * n + q) * jprev + jp) * in_ld + f], y);
+            out[(r * jout + to) * out_ld + f] = y;
         }
     }
 }

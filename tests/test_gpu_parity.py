@@ -1607,3 +1607,38 @@ def test_sparse_grid_projection_of_few_fields_takes_the_shorter_chain():
     assert _device_us(lambda: e.project(few, c)) < 1.3 * _device_us(lambda: e.project_block(few, 0, c))
     assert _device_us(lambda: e.project(m, whole)) < 0.6 * _device_us(lambda: e.project_block(m, 0, whole))
     e.close()
+
+
+@pytest.mark.parametrize("dim,order,pts,quad", [(1, 1, 2, 0), (1, 4, 5, 0), (2, 3, 4, 0), (3, 4, 5, 0), (2, 8, 9, 0),
+                                                (1, 2, 2, 1), (2, 3, 3, 1), (4, 3, 3, 1)])
+def test_projection_of_values_near_the_largest_number(dim, order, pts, quad):
+    """FP64 fields of 0.95e308, whose sums or differences over opposite points leave the range while the
+    coefficients do not: constants and odd fields on tensor grids, and on sparse grids one pair of opposite
+    samples (weights below a half) with equal and with opposite signs.  Against the dense contraction, to S
+    roundings 2^-53 of sum |W| |M| on either side, and on sparse grids to the 1e-13 of a term's largest weight
+    within which the plan takes the weights of reflected samples for equal."""
+    e = Ensemble(0)
+    e.set_inputs([(-1.0, 1.0)] * dim)
+    U.uqlb_init_gpc(e.ctx, order, pts, 0, quad)
+    S, K = e.num_samples, e.num_terms
+    _, xi, _ = U.uqlb_get_samples(e.ctx, dim)
+    big = 0.95e308
+    m = np.zeros((S, 50000))  # many fields, so that the sparse grids go over reflected samples
+    if quad == 0:
+        m[:, 0] = big
+        m[:, 1] = big * np.sign(xi[:, 0])
+        m[:, 2] = -big
+    else:
+        on_axis = [i for i in range(S) if np.abs(xi[i, 1:]).sum() < 1e-12]
+        s = next(i for i in on_axis if xi[i, 0] > 1e-12)
+        o = next(i for i in on_axis if abs(xi[i, 0] + xi[s, 0]) < 1e-12)
+        m[s, :3], m[o, 0], m[o, 1], m[o, 2] = big, big, -big, 0.0
+    m[:, -1] = np.arange(S)
+    t = torch.from_numpy(m).cuda()
+    got, dense = e.project(t).cpu().numpy(), e.project_block(t, 0).cpu().numpy()
+    assert np.isfinite(dense).all()
+    at = [0, 1, 2, -1]
+    w, x = np.abs(U.uqlb_get_weight_matrix(e.ctx)), np.abs(m[:, at]) * 1e-10
+    bound = 2 * S * 2.0 ** -53 * (w @ x) + (1e-13 * w.max(axis=1)[:, None] * x.sum(axis=0) if quad else 0.0)
+    assert np.all(np.abs(got[:, at] * 1e-10 - dense[:, at] * 1e-10) <= bound)
+    e.close()
