@@ -414,15 +414,9 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
         const int n_mine = have ? min(p.spl, steps - t) : 0;
 
         const int n_max = __reduce_max_sync(kAll, n_mine);
-        // a sample records if one of its own steps of this launch is a recorded one: every warp that holds
-        // it has to come to the same answer (its counter below waits for all of them), whatever other
-        // samples the warp holds
-        auto records = [&](int n) {
-            bool any = false;
-            for (int k = 0; k < n; ++k) any = any || (t + k) % p.qoi_every == 0;
-            return any;
-        };
-        const bool rec = series && records(n_max);
+        bool rec = false;
+        if (series)
+            for (int k = 0; k < n_max; ++k) rec = rec || (t + k) % p.qoi_every == 0;
         double red[NS];
 #pragma unroll
         for (int k = 0; k < NS; ++k) red[k] = 0.0;
@@ -440,7 +434,10 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
         // in a fixed order by the last warp of a sample to finish
         for (int c = 0; c < T; ++c) {
             if (m * T + c >= nact) break;
-            if (!records(min(p.spl, p.samples[m * T + c].steps - t))) continue;
+            // a sample is summed if one of its own steps of this launch is a recorded one: every warp that holds
+            // it has to come to the same answer (its counter waits for all of them), whatever other samples the
+            // warp holds
+            if ((p.qoi_every - t % p.qoi_every) % p.qoi_every >= min(p.spl, p.samples[m * T + c].steps - t)) continue;
             uint64_t warps = 0;  // the group's warps that hold useful columns of task c
             if (map.closed) {
                 warps = 1;
