@@ -325,8 +325,10 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
     const int nx = W > 0 ? W : map.nx;
     const int U = (nx + 1) >> 1;
 
-    // this lane's sample within the group of T (task), column pair and neighbours
-    int task = -1, px = 0, left = (lane + 31) & 31, right = (lane + 1) & 31;
+    // this lane's sample within the group of T (task), column pair and neighbours.  Idle lanes load pairs of
+    // their own too: all on one pair, its copies into their slots came one after the other (1 x 57 x 33: 2.48
+    // against 1.93 us per step, 1 x 512^2 3.15 / 2.78, 16 x 97^2 2.97 / 2.76)
+    int task = -1, px = lane % U, left = (lane + 31) & 31, right = (lane + 1) & 31;
     bool useful = false;
     if (map.closed) {
         if (lane / U < T) {

@@ -1642,3 +1642,14 @@ def test_projection_of_values_near_the_largest_number(dim, order, pts, quad):
     bound = 2 * S * 2.0 ** -53 * (w @ x) + (1e-13 * w.max(axis=1)[:, None] * x.sum(axis=0) if quad else 0.0)
     assert np.all(np.abs(got[:, at] * 1e-10 - dense[:, at] * 1e-10) <= bound)
     e.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+def test_idle_lanes_of_the_register_strips_cost_nothing(ens, storage):
+    """Rows of 57 columns leave 27 of a warp's lanes idle, rows of 47 four: one sample of either is a chain of
+    the same length, so the times are alike (idle lanes that all load one pair made it a fifth longer)."""
+    def us(nx):
+        samples, out = [sample_struct(replace(W.tgv(nx, 2000, nu=0.04), ny=33))], {}
+        return _device_us(lambda: ens.run_batch(samples, storage=storage, out=out, scheme="three_step_strips"))
+
+    assert us(57) < 1.1 * us(47)
