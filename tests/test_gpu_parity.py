@@ -1653,3 +1653,67 @@ def test_idle_lanes_of_the_register_strips_cost_nothing(ens, storage):
         return _device_us(lambda: ens.run_batch(samples, storage=storage, out=out, scheme="three_step_strips"))
 
     assert us(57) < 1.1 * us(47)
+
+
+@pytest.mark.parametrize("storage", ["f16", "bf16", "fx16"])
+@pytest.mark.parametrize("nx,ny,n", [(31, 31, 3), (33, 40, 4), (57, 29, 5), (62, 33, 3), (63, 64, 1), (66, 50, 4), (113, 60, 3),
+                                     (127, 127, 2), (255, 64, 3), (256, 40, 3), (300, 48, 2), (48, 48, 4)])
+def test_register_strips_of_16_bit_lattices_equal_the_two_step_strips(ens, storage, nx, ny, n):
+    """16-bit lattices that keep their flow, samples of their own amplitude side by side: runs of two steps,
+    each resumed by the next, round once per two steps on either kernel, so that states, fields and sums of
+    eight steps are the same collisions and the same roundings (to nearest): equal bit for bit (K sums in
+    another order).  A wrong halo, seam or neighbouring sample shows in velocities above a hundredth."""
+    specs = [replace(W.tgv(nx, 8, nu=0.01, u0=0.02 + 0.004 * k, amp2=0.002 * (k + 1), amp3=-0.003), ny=ny)
+             for k in range(n)]
+
+    def run(scheme):
+        for step in range(0, 8, 2):
+            batch = [sample_struct(replace(s, steps=step + 2)) for s in specs]
+            res = ens.run_batch(batch, storage=storage, rounding="nearest", scheme=scheme, start_step=step)
+        torch.cuda.synchronize()
+        return {k: v.double().cpu().numpy() for k, v in res.items()}
+
+    a, b = run("two_step_strips"), run("three_step_strips")
+    assert np.array_equal(b["fields"][:, :-1], a["fields"][:, :-1])
+    assert np.allclose(b["fields"][:, -1], a["fields"][:, -1], rtol=2.0 ** -22, atol=0)
+    assert all(np.abs(f[:-1]).max() > 0.01 for f in a["fields"])
+    assert len({round(float(f[-1]), 6) for f in a["fields"]}) == n
+
+
+@pytest.mark.parametrize("storage", ["f16", "bf16", "fx16"])
+@pytest.mark.parametrize("nx,ny,n", [(31, 31, 3), (33, 40, 4), (57, 29, 5), (62, 33, 3), (63, 64, 1), (66, 50, 4),
+                                     (113, 60, 3), (48, 48, 4)])
+def test_register_strips_of_16_bit_lattices_over_one_whole_launch(ens, storage, nx, ny, n):
+    """Three steps, the whole of a 16-bit launch, against the FP32 strips: the start and the launch round every
+    population once, each by half a step of its format (F16 2^-11, BF16 2^-8 of a population below U/3 + 3 U^2,
+    U the largest speed; FX16 its quantum), and u sums at most nine of them over rho near 1, 2 x 9 x step / 2.
+    That is at most a tenth of the velocities, and less than what a swap of columns changes."""
+    specs = [replace(W.tgv(nx, 3, nu=0.01, u0=0.02 + 0.004 * k, amp2=0.002 * (k + 1), amp3=-0.003), ny=ny)
+             for k in range(n)]
+    f32 = _run(ens, specs, "f32", scheme="three_step_strips")["fields"][:, :-1]
+    res = ens.run_batch([sample_struct(s) for s in specs], storage=storage, rounding="nearest", scheme="three_step_strips")
+    torch.cuda.synchronize()
+    got = res["fields"].double().cpu().numpy()[:, :-1]
+    assert np.all(res["qoi"].cpu().numpy()[:, U.UQLB_QOI_STATUS] == 0)
+    for i, s in enumerate(specs):
+        top = np.abs(f32[i]).max()
+        if storage == "fx16":
+            step = float(U.uqlb_fx16_quanta(sample_struct(s)).max())
+        else:
+            step = (top / 3 + 3 * top ** 2) * 2.0 ** (-11 if storage == "f16" else -8)
+        bound = 2 * 9 * step / 2
+        assert bound < 0.1 * top
+        u = f32[i][: nx * ny].reshape(ny, nx)
+        assert np.abs(np.diff(u, axis=1)).max() > bound
+        assert np.abs(got[i] - f32[i]).max() <= bound, i
+
+
+def test_fp64_collision_conserves_mass(ens):
+    """20000 steps of a fast flow that hardly decays: the coefficients of the collision's quadratic term sum to
+    zero as rounded, so that the mass walks by single roundings only, some 1e-17 of it (256^2 nodes x 20000
+    steps x 18 roundings of 2^-54 of populations near 0.03, in quadrature).  A sum of 2^-53 is a gain of
+    2^-53 omega j^2 / 2 per node and step, 8e-15 here."""
+    s = W.tgv(256, 20000, nu=0.0088, u0=0.1)
+    start, end = (_run(ens, [replace(s, steps=k)], "f64")["qoi"][0] for k in (0, s.steps))
+    assert end[U.UQLB_QOI_K] > 0.5 * start[U.UQLB_QOI_K]
+    assert abs(end[U.UQLB_QOI_MASS] - start[U.UQLB_QOI_MASS]) < 1e-15 * start[U.UQLB_QOI_MASS]
