@@ -366,22 +366,35 @@ __device__ __forceinline__ bool sf_group(const TI* src, int64_t step, const doub
 }
 
 // The same for n points that are not compiled in, without the fold: the inputs are loaded and converted once,
-// and the degrees are CNT independent chains, eight inputs in flight (four lose 11 % at five degrees and 10
-// points, gain 7 % at two).  Measured with the statistics, FP32 / FP64 fields, 131073 fields: 16 x 16 points at
-// degree 8 756 / 678 us, 10 x 10 at degree 4 195 / 167; one degree after the other, which reloads and
-// converts the inputs for each, 1288 / 681 and 296 / 168; all nine degrees with predicates 887 / 813, 357 / 329.
+// and the degrees are CNT independent chains, with eight, four, two and one inputs in flight (n = 10 in fours
+// with a remainder one by one: 12 % longer).  Measured with the statistics, FP32 / FP64 fields, 131073 fields:
+// 16 x 16 points at degree 8 757 / 682 us, 10 x 10 at degree 4 195 / 167; one degree after the other, which
+// reloads and converts the inputs for each, 1288 / 682 and 296 / 167; all nine degrees with predicates 887 / 813
+// and 357 / 329.
 template <int CNT, typename TI>
 __device__ __forceinline__ void sf_group_any(const TI* src, int64_t step, int n, const double (*G)[kSfMaxPoints],
                                              double* out, int64_t out_ld, const int* __restrict__ o) {
     double y[CNT];
 #pragma unroll
     for (int a = 0; a < CNT; ++a) y[a] = 0.0;
-#pragma unroll (CNT <= 2 ? 4 : 8)
-    for (int q = 0; q < n; ++q) {
-        const double x = (double)src[q * step];
+    int q = 0;
+    auto take = [&](auto u_c) {
+        constexpr int U = decltype(u_c)::value;
+        TI v[U];
 #pragma unroll
-        for (int a = 0; a < CNT; ++a) y[a] = fma(G[a][q], x, y[a]);
-    }
+        for (int i = 0; i < U; ++i) v[i] = src[(q + i) * step];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const double x = (double)v[i];
+#pragma unroll
+            for (int a = 0; a < CNT; ++a) y[a] = fma(G[a][q + i], x, y[a]);
+        }
+        q += U;
+    };
+    while (n - q >= 8) take(std::integral_constant<int, 8>{});
+    if (n - q >= 4) take(std::integral_constant<int, 4>{});
+    if (n - q >= 2) take(std::integral_constant<int, 2>{});
+    if (n - q >= 1) take(std::integral_constant<int, 1>{});
 #pragma unroll
     for (int a = 0; a < CNT; ++a) out[(int64_t)__ldg(o + a) * out_ld] = y[a];
 }
