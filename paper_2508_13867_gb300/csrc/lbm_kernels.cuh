@@ -2637,12 +2637,13 @@ StripBlocks strip_blocks_of(K kernel, int threads, size_t dyn, int default_kb) {
     return r;
 }
 
-// Blocks per SM of one instantiation of the three-step strips (once).  By default the most blocks that
+// Blocks per SM of one instantiation of the three-step strips (once; of the kernel with series, which takes no
+// fewer registers than the one without).  By default the most blocks that
 // fit and the smallest shared-memory share that holds them: the rest of the 256 KB is L1, where the
 // halo columns that neighbouring windows share are found.
 template <typename S, int W, int D, bool ODD>
 const StripBlocks& strip_regs_blocks() {
-    static const StripBlocks b = strip_blocks_of(strip_regs_kernel<S, W, D, ODD>, kStripThreads, 0, -1);
+    static const StripBlocks b = strip_blocks_of(strip_regs_kernel<S, W, D, ODD, true>, kStripThreads, 0, -1);
     return b;
 }
 
@@ -2691,6 +2692,8 @@ cudaError_t launch_strip_regs_d(const KParams& p, const BatchGeometry& g, cudaSt
         while (k.next()) {
             map.stretch[n++] = {(uint8_t)k.task, (uint8_t)k.lane0, (uint8_t)k.count, 0, k.first};
             map.start[k.warp + 1] = (uint8_t)n;
+            if (k.first == 0) map.first_warp[k.task] = (uint8_t)k.warp;
+            map.warps_of[k.task] = (uint8_t)(k.warp + 1 - map.first_warp[k.task]);
         }
     }
     int bps = 0, kb = 0;
@@ -2715,7 +2718,9 @@ cudaError_t launch_strip_regs_d(const KParams& p, const BatchGeometry& g, cudaSt
     at[0].val.sharedMemCarveout = (unsigned)carveout_pct(kb);
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, strip_regs_kernel<S, W, D, ODD>, p, map);
+    if (p.qoi_every > 0 && p.series != nullptr)
+        return cudaLaunchKernelEx(&cfg, strip_regs_kernel<S, W, D, ODD, true>, p, map);
+    return cudaLaunchKernelEx(&cfg, strip_regs_kernel<S, W, D, ODD, false>, p, map);
 }
 
 // Staging of a launch's phase-0 rows: option 1 = none, 2 = the next rows in shared memory by cp.async,

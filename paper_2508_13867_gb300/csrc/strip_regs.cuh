@@ -237,14 +237,20 @@ __device__ __forceinline__ void strip_piece(const KParams& p, const StripPiece<S
         auto collide = [&](f2(&h)[9], int k) {
             if constexpr (REC) {
                 const int row = it - k - (n - 1);
-                if (want[k] && put && row >= 0 && row < L) {
-                    f2 q;
+                // one branch for the warp: on `put` as well, halo and useful lanes would collide one after
+                // the other.  Odd widths form u.u in every phase, whose one copy of the collision leaves
+                // the other rows' code better off (128 x 127^2 with a series every 100 steps 11.81 against
+                // 11.92 us per step; 625 x 256^2 130.3 against 127.8)
+                f2 q;
+                const bool sum = want[k] && row >= 0 && row < L;
+                if (ODD || sum)
                     collide_packed(h, om, &q);
+                else
+                    collide_packed(h, om, nullptr);
+                if (sum && put) {
                     float a, b;
                     upk(q, a, b);
                     red[k] += (double)a + (use_b ? (double)b : 0.0);
-                } else {
-                    collide_packed(h, om, nullptr);
                 }
             } else {
                 // FP32: the last two phases in scalar instructions (the same bits), which balances the
@@ -304,10 +310,116 @@ __device__ __forceinline__ void strip_piece(const KParams& p, const StripPiece<S
     }
 }
 
+// Sums of NS <= 4 values over the warp, value k in the lanes 8 k of the result: at the first two levels a lane
+// keeps half of the values and sends the others (6 FP64 adds instead of 5 NS, whose units all warps share),
+// in the order of one butterfly per value.
+template <int NS>
+__device__ __forceinline__ double strip_warp_sums(const double (&v)[NS], int lane) {
+    static_assert(NS == 3 || NS == 4, "two levels of halves");
+    const bool hi = (lane & 16) != 0, odd = (lane & 8) != 0;
+    const double v3 = NS == 4 ? v[NS - 1] : 0.0;
+    const double a = (hi ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
+    const double b = (hi ? v3 : v[1]) + __shfl_xor_sync(0xffffffffu, hi ? v[1] : v3, 16);
+    double r = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    return r;
+}
+
+// Sum over the warp of n slots of one sample: `nw` consecutive warps of every piece, G T NS apart.  Eight
+// slots of a lane are in flight at once.  Not inlined: its registers are its own, not the row loop's.
+template <int NS>
+__device__ __noinline__ double strip_slots_sum(const double* slots, int n, int nw, int G, int T) {
+    constexpr int kAhead = 8;
+    const int lane = threadIdx.x & 31;
+    double acc[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) acc[k] = 0.0;
+    for (int q0 = lane; q0 < n; q0 += 32 * kAhead) {
+        double v[kAhead][NS];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            const int q = q0 + 32 * i, at = q / nw;
+            const double* from = slots + ((int64_t)at * G + (q - at * nw)) * T * NS;
+#pragma unroll
+            for (int k = 0; k < NS; ++k) v[i][k] = q < n ? __ldcg(from + k) : 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i)
+#pragma unroll
+            for (int k = 0; k < NS; ++k) acc[k] += v[i][k];
+    }
+    return strip_warp_sums<NS>(acc, lane);
+}
+
+// What the sums of a piece need besides the kernel's parameters.
+struct StripSums {
+    const SampleDev* samples;
+    double *kpart, *series;
+    int32_t* counters;
+    int64_t qoi_every, series_ld;
+    int spl, t, nact, T, G, slot, task, m, ny, rb, ya, yb, per, parts, group;
+};
+
+// K: the warp's sum of each of its tasks into the slot of (range, warp, sample); the last warp of a sample to
+// finish sums its slots in a fixed order.  The warp's tasks share one fence, which waits for the rows' stores
+// too, and count in parallel, a lane each.  Three 256 x 256 samples with the energy of every step, us per
+// step: FP32 6.9, FX16 8.3 (2.7 and 3.4 without); with a fence, a count and a butterfly per value for each
+// task, one slot after the other and halo lanes that collided apart from the others 13.4 and 20.0.
+template <int NS>
+__device__ __forceinline__ void strip_record(const StripSums& a, const StripMap& map, const double (&red)[NS]) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    // Lane c looks after task c.  A sample is summed if one of its own steps of this launch is a recorded one:
+    // every warp that holds it has to come to the same answer (its counter waits for all of them),
+    // whatever other samples the warp holds.
+    const int64_t wait = (a.qoi_every - a.t % a.qoi_every) % a.qoi_every;  // steps from t to the next recorded one
+    const int mine = a.m * a.T + lane;
+    int w0 = 0, nw = 0;  // the group's warps that hold columns of the task
+    if (lane < a.T && mine < a.nact && wait < min(a.spl, a.samples[mine].steps - a.t)) {
+        nw = map.closed ? 1 : map.warps_of[lane];
+        w0 = map.closed ? 0 : map.first_warp[lane];
+    }
+    const unsigned held = __ballot_sync(kAll, a.slot >= w0 && a.slot < w0 + nw);
+    // pieces are numbered along the ranges: a piece is one range's part of one group of samples
+    const int piece = a.parts > 0 ? a.group : a.m + a.group;
+    for (unsigned left = held; left != 0; left &= left - 1) {
+        const int c = __ffs(left) - 1;
+        double part[NS];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) part[k] = a.task == c ? red[k] : 0.0;
+        const double sum = strip_warp_sums<NS>(part, lane);
+        if ((lane & 7) == 0 && lane / 8 < NS)
+            a.kpart[(((int64_t)piece * a.G + a.slot) * a.T + c) * NS + lane / 8] = sum;
+    }
+    __threadfence();
+    __syncwarp();
+    bool last = false;
+    if ((held >> lane) & 1) last = atomicAdd(a.counters + mine, a.yb - a.ya) + (a.yb - a.ya) == a.ny * nw;
+    const unsigned done = __ballot_sync(kAll, last);
+    if (done == 0) return;
+    __threadfence();
+    const int first = a.parts > 0 ? a.m * a.parts : a.m + a.rb / a.per;
+    const int pieces = a.parts > 0 ? a.parts : (a.rb + a.ny - 1) / a.per - a.rb / a.per + 1;
+    for (unsigned left = done; left != 0; left &= left - 1) {
+        const int c = __ffs(left) - 1, jc = a.m * a.T + c;
+        const int cw0 = __shfl_sync(kAll, w0, c), cnw = __shfl_sync(kAll, nw, c);
+        const double* slots = a.kpart + (((int64_t)first * a.G + cw0) * a.T + c) * NS;
+        const double total = strip_slots_sum<NS>(slots, pieces * cnw, cnw, a.G, a.T);
+        const SampleDev* sc = a.samples + jc;
+        const int k = lane / 8;
+        if ((lane & 7) == 0 && k < min(a.spl, sc->steps - a.t) && (a.t + k) % a.qoi_every == 0)
+            a.series[(int64_t)sc->sample_id * a.series_ld + (a.t + k) / a.qoi_every] = total * sc->u_ref_inv2;
+        if (lane == 0) a.counters[jc] = 0;
+    }
+}
+
 // W: compile-time width (0: map.nx; 256 columns 564 instead of 527 us per launch).  D: the phase-0 row is
 // loaded when it is used (0), kStripDepth rows ahead into shared memory by cp.async (1) or one row ahead
-// into registers (2).  ODD: odd widths.
-template <typename S, int W, int D, bool ODD>
+// into registers (2).  ODD: odd widths.  SERIES: launches of runs that record K at some step; the others' kernel
+// holds no second copy of the rows' code with its sums (625 x 256^2 124.9 against 125.7 us per step, 1 x 128^2 1.52
+// / 1.69, FX16 128 x 256^2 38.2 / 39.5).
+template <typename S, int W, int D, bool ODD, bool SERIES>
 __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) strip_regs_kernel(KParams p, const __grid_constant__ StripMap map) {
     static_assert(!ODD || D == 1, "unaligned pairs are put together in shared memory");
     constexpr int NS = kStripSteps<S>;
@@ -366,7 +478,6 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
     const int per = parts > 0 ? map.part : (rows + ngroups - 1) / ngroups;
     const int r0 = parts > 0 ? group / parts * map.ny + group % parts * per : group * per;
     const int r1 = parts > 0 ? min(min(rows, r0 + per), (group / parts + 1) * map.ny) : min(rows, r0 + per);
-    const bool series = p.qoi_every > 0 && p.series != nullptr;
 
     for (int r = r0; r < r1;) {
         int m, rb, ny;
@@ -417,7 +528,7 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
 
         const int n_max = __reduce_max_sync(kAll, n_mine);
         bool rec = false;
-        if (series)
+        if (SERIES)
             for (int k = 0; k < n_max; ++k) rec = rec || (t + k) % p.qoi_every == 0;
         double red[NS];
 #pragma unroll
@@ -426,77 +537,17 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
         for (int n = n_max; n >= 1; --n) {
             if (!__any_sync(kAll, n_mine == n)) continue;
             const bool put = useful && n_mine == n;
-            if (rec)
+            if (SERIES && rec)
                 strip_piece<S, D, ODD, true>(p, pc, stage, t, n, put, red);
             else
                 strip_piece<S, D, ODD, false>(p, pc, stage, t, n, put, red);
         }
-        if (!rec) continue;
-        // K: the warp's sum of each of its tasks into the slot of (range, sample, warp, task), summed
-        // in a fixed order by the last warp of a sample to finish
-        for (int c = 0; c < T; ++c) {
-            if (m * T + c >= nact) break;
-            // a sample is summed if one of its own steps of this launch is a recorded one: every warp that holds
-            // it has to come to the same answer (its counter waits for all of them), whatever other samples the
-            // warp holds
-            if ((p.qoi_every - t % p.qoi_every) % p.qoi_every >= min(p.spl, p.samples[m * T + c].steps - t)) continue;
-            uint64_t warps = 0;  // the group's warps that hold useful columns of task c
-            if (map.closed) {
-                warps = 1;
-            } else {
-                for (int w = 0; w < G; ++w)
-                    for (int q = map.start[w]; q < map.start[w + 1]; ++q)
-                        if (map.stretch[q].task == c) warps |= 1ull << w;
-            }
-            if (!((warps >> slot) & 1)) continue;
-            const int jc = m * T + c;
-            double part[NS];
+        if (!SERIES || !rec) continue;
+        double sums[NS];
 #pragma unroll
-            for (int k = 0; k < NS; ++k) {
-                part[k] = task == c ? red[k] : 0.0;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) part[k] += __shfl_xor_sync(kAll, part[k], o);
-            }
-            // pieces are numbered along the ranges: a piece is one range's part of one group of samples
-            const int piece = parts > 0 ? group : m + group;
-            int last = 0;
-            if (lane == 0) {
-                double* to = p.kpart + ((((int64_t)piece * G + slot) * T + c) * NS);
-#pragma unroll
-                for (int k = 0; k < NS; ++k) to[k] = part[k];
-                __threadfence();
-                const int goal = ny * __popcll(warps);
-                last = atomicAdd(p.counters + jc, yb - ya) + (yb - ya) == goal;
-            }
-            last = __shfl_sync(kAll, last, 0);
-            if (!last) continue;
-            __threadfence();
-            const int first = parts > 0 ? m * parts : m + rb / per;
-            const int pieces = parts > 0 ? parts : (rb + ny - 1) / per - rb / per + 1;
-            double acc[NS];
-#pragma unroll
-            for (int k = 0; k < NS; ++k) acc[k] = 0.0;
-            for (int q = lane; q < pieces * G; q += 32) {
-                const int s = q % G, at = first + q / G;
-                if (!((warps >> s) & 1)) continue;
-                const double* from = p.kpart + ((((int64_t)at * G + s) * T + c) * NS);
-#pragma unroll
-                for (int k = 0; k < NS; ++k) acc[k] += __ldcg(from + k);
-            }
-#pragma unroll
-            for (int k = 0; k < NS; ++k)
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(kAll, acc[k], o);
-            if (lane == 0) {
-                const SampleDev* sc = p.samples + jc;
-                const int n_c = min(p.spl, sc->steps - t);
-                const int64_t row = (int64_t)sc->sample_id * p.series_ld;
-#pragma unroll
-                for (int k = 0; k < NS; ++k)
-                    if (k < n_c && ((t + k) % p.qoi_every) == 0)
-                        p.series[row + (t + k) / p.qoi_every] = acc[k] * sc->u_ref_inv2;
-                p.counters[jc] = 0;
-            }
-        }
+        for (int k = 0; k < NS; ++k) sums[k] = red[k];
+        const StripSums a{p.samples, p.kpart, p.series, p.counters, p.qoi_every, p.series_ld, p.spl, t, nact, T, G,
+                          slot, task, m, ny, rb, ya, yb, per, parts, group};
+        strip_record<NS>(a, map, sums);
     }
 }

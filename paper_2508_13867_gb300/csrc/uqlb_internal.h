@@ -239,8 +239,10 @@ struct StripMap {
     int32_t samples, warps, closed, nx, ny;  // ny: common height (0: heights differ)
     int32_t part;  // rows of one group of samples per range (0: equal ranges over all rows)
     uint8_t start[kStripGroupWarps + 4];
+    uint8_t first_warp[8], warps_of[8];  // the consecutive warps that hold columns of a sample (rows that do not close)
     StripStretch stretch[kStripGroupWarps + kStripGroupSamples];
 };
+static_assert(kStripGroupSamples <= 8, "first_warp and warps_of");
 // Three-step strips of batch g at staging option `stage` (1: none, 2: one row, 0: default): the
 // most resident blocks per SM, the default, the default shared-memory share (KB) and the shared
 // memory per block (bytes).  False when g does not run on the three-step strips or the staging

@@ -1717,3 +1717,17 @@ def test_fp64_collision_conserves_mass(ens):
     start, end = (_run(ens, [replace(s, steps=k)], "f64")["qoi"][0] for k in (0, s.steps))
     assert end[U.UQLB_QOI_K] > 0.5 * start[U.UQLB_QOI_K]
     assert abs(end[U.UQLB_QOI_MASS] - start[U.UQLB_QOI_MASS]) < 1e-15 * start[U.UQLB_QOI_MASS]
+
+
+@pytest.mark.parametrize("storage", ["f32", "fx16"])
+def test_energy_series_of_every_step_in_the_register_strips(ens, storage):
+    """Three 256 x 256 samples with the energy of every step: many warps hold parts of a sample, and their sums are
+    on every launch's path.  No longer than the two-step strips, whose blocks hold whole rows, by more than a
+    half (parts summed one after the other took two to three times as long)."""
+    samples = [sample_struct(W.tgv(256, 400, nu=0.03)) for _ in range(3)]
+    us = {}
+    for scheme in ("three_step_strips", "two_step_strips"):
+        out = {}
+        us[scheme] = _device_us(lambda: ens.run_batch(samples, storage=storage, qoi_every=1, series=True, out=out,
+                                                      scheme=scheme))
+    assert us["three_step_strips"] < 1.5 * us["two_step_strips"]
