@@ -38,7 +38,7 @@ STEP_KERNELS = {1: ("step_kernel (one-step: fused AA collide-stream-QoI, in plac
                     "and collided again, pushed to the other lattice)", "strip2_kernel", "two-step-strips-v2-staged"),
                 6: ("strip_regs_kernel (row strips with three or four steps per launch: each warp walks a window of "
                     "64 columns down its rows and keeps the rows between the steps in registers)", "strip_regs_kernel",
-                    "strips-in-registers-v1")}
+                    "strips-in-registers-v2")}
 
 
 def steps_per_launch_of(scheme: int, storage: str) -> int:

@@ -562,7 +562,7 @@ int uqlb_project_noalloc(uqlb_ctx* ctx, const void* m_dev, int dtype, int64_t n_
  *     coeffs_dev: FP64 [K x n_fields]; the workspace is uqlb_post_workspace_bytes.  Synchronises
  *     `stream` after the weight upload.  UQLB_ERR_ARG for a block outside 0 .. S - 1.
  *   MC: uqlb_block_moments gives the block's mean[f] (Eq. meanMCS over its n_rows rows) and
- *     m2[f] = sum over the rows of (M[s, f] - mean[f])^2 (two passes, FP64); blocks merge exactly by the
+ *     m2[f] = sum over the rows of (M[s, f] - mean[f])^2 (as uqlb_stats forms them); blocks merge exactly by the
  *     pairwise update of Chan, Golub and LeVeque (n = n_a + n_b, delta = mean_b - mean_a,
  *     mean = mean_a + delta n_b / n, m2 = m2_a + m2_b + delta^2 n_a n_b / n), and Eq. varMCS is
  *     m2 / (N - ddof).  The call needs no sample set (any context serves).
@@ -578,7 +578,11 @@ int uqlb_block_moments(uqlb_ctx* ctx, const void* m_dev, int dtype, int64_t n_ro
  *   gPC context: input is coeffs_dev [K x n_fields] FP64; mean = c_0 (Eq. gpc_mean),
  *     var = sum_{k >= 1} c_k^2 (Eq. gpc_std squared); dtype must be UQLB_F64, ddof ignored.
  *   MC context: input is M [S x n_fields] (ld = m_ld) in `dtype`; mean by Eq. meanMCS,
- *     var by Eq. varMCS with divisor S - ddof (two passes, FP64). */
+ *     var by Eq. varMCS with divisor S - ddof.  FP64 fields, and FP32 fields of few samples: two passes in
+ *     FP64.  FP32 fields of many samples: one pass over the deviations from the field's first sample, which
+ *     FP32 pairs hold exactly, with their sum and the sum of their squares as sums of three FP32 numbers
+ *     (about 70 bits) and the last step in pairs of FP64 numbers; fields with a non-finite value or a
+ *     deviation outside [1e-15, 1e15] in two passes. */
 int uqlb_stats(uqlb_ctx* ctx, const void* in_dev, int dtype, int64_t n_fields, int64_t m_ld,
                double* mean_dev, double* var_dev, int ddof, void* stream);
 

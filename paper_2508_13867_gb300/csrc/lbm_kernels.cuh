@@ -1826,8 +1826,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) cluster_kernel(KParams p) 
                     gather_odd(k, yn, xn, own, lw, v);
 #pragma unroll
                     for (int i = 0; i < 9; ++i) g[i] = Storage<S>::load(v + i, qz, i);
-    
-    } else {
+                } else {
 #pragma unroll
                     for (int i = 0; i < 9; ++i) g[i] = Storage<S>::load(lat + own + i * RC, qz, i);
                 }
@@ -2638,9 +2637,9 @@ StripBlocks strip_blocks_of(K kernel, int threads, size_t dyn, int default_kb) {
 }
 
 // Blocks per SM of one instantiation of the three-step strips (once; of the kernel with series, which takes no
-// fewer registers than the one without).  By default the most blocks that
-// fit and the smallest shared-memory share that holds them: the rest of the 256 KB is L1, where the
-// halo columns that neighbouring windows share are found.
+// fewer registers than the one without).  By default the most blocks that fit and the smallest shared-memory
+// share that holds them: the rest of the 256 KB is L1, where the halo columns that neighbouring windows
+// share are found.
 template <typename S, int W, int D, bool ODD>
 const StripBlocks& strip_regs_blocks() {
     static const StripBlocks b = strip_blocks_of(strip_regs_kernel<S, W, D, ODD, true>, kStripThreads, 0, -1);
@@ -2718,7 +2717,14 @@ cudaError_t launch_strip_regs_d(const KParams& p, const BatchGeometry& g, cudaSt
     at[0].val.sharedMemCarveout = (unsigned)carveout_pct(kb);
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (p.qoi_every > 0 && p.series != nullptr)
+    // FP32 lattices of odd width beyond half a gigabyte run faster on the code of the kernel with series, whose
+    // registers spill more (us per step with / without: 400 x 255^2 94.4 / 95.9, 630 x 255^2 148 / 154, 500 x 201^2
+    // 88.9 / 95.6, 400 x 313^2 164 / 186, 2000 x 127^2 126 / 131); below that, and with 16-bit storage, they do
+    // not (200 x 255^2 49.0 / 48.6, 300 x 127^2 21.7 / 21.3, 5 x 97^2 2.22 / 2.12, BF16 630 x 255^2 187 / 181).
+    // The instructions are the same; the time follows the lattice's size.
+    const int64_t lattice = (int64_t)g.total_rows * 18 * strip_threads(g.strip_nx) * (int64_t)sizeof(S);
+    const bool big_odd = ODD && sizeof(S) == 4 && lattice > ((int64_t)1 << 29);
+    if ((p.qoi_every > 0 && p.series != nullptr) || big_odd)
         return cudaLaunchKernelEx(&cfg, strip_regs_kernel<S, W, D, ODD, true>, p, map);
     return cudaLaunchKernelEx(&cfg, strip_regs_kernel<S, W, D, ODD, false>, p, map);
 }

@@ -220,7 +220,7 @@ __device__ __forceinline__ void add(Sum3& s, const Sum3& x) {
 struct Pair64 {
     double h, l;
 };
-__device__ __forceinline__ Pair64 quick_sum(double a, double b) {  // |a| >= |b|, or a == 0
+__device__ __forceinline__ Pair64 quick_sum(double a, double b) {  // Dekker's fast two-sum: |a| >= |b|, or a == 0
     const double h = a + b;
     return {h, b - (h - a)};
 }

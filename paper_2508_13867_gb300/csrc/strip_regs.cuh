@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(kStripThreads, kStripMinBlocks<S, D, ODD>) str
 
         const int n_max = __reduce_max_sync(kAll, n_mine);
         bool rec = false;
-        if (SERIES)
+        if (SERIES && p.qoi_every > 0 && p.series != nullptr)
             for (int k = 0; k < n_max; ++k) rec = rec || (t + k) % p.qoi_every == 0;
         double red[NS];
 #pragma unroll

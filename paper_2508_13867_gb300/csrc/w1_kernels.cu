@@ -12,8 +12,8 @@
 // FP64 instructions issue at 1/75 of the FP32 rate on GB300, and these kernels have nothing else to wait
 // for, so they use FP64 only where FP32 cannot decide:
 //   largest speed: the squared speed in FP32 picks the candidates, FP64 decides between close ones;
-//   bins: the speed as the sum of two FP32 numbers (error below 2^-40 of it) gives the bin unless the
-//     speed lies that close to an edge; then the FP64 formula decides;
+//   bins: the speed as the sum of two FP32 numbers (error below 2^-42 of it) gives the bin unless the
+//     speed lies close to an edge (2^-40 of the range and a little more); then the FP64 formula decides;
 //   distance: sum |n_b C_a - n_a C_b| over the bins in integers (C: cumulative counts; 64-bit products,
 //     128-bit sum), one division at the end.
 // Measured on 128 x 127^2 and 256 x 255^2 FP32 speeds in 2^20 bins: 0.30 against 7.83 ms in all (two
@@ -78,8 +78,8 @@ __global__ void __launch_bounds__(kThreads) max_speed_kernel(const M* m, int64_t
 
 // Bin of the speed of (u, v) under scale = sh + sl bins per unit, as FP32 pairs: u^2 + v^2 with its
 // rounding errors, the root by one Newton step on the approximate one, times the scale.  All errors
-// together stay below 2^-42 of the result; false where the result lies within delta = 2^-40 bins of an
-// edge (or outside FP32's range, or is not finite) and FP64 has to decide.
+// together stay below 2^-42 of the result, which is at most `bins`; false where the result lies within delta =
+// bins 2^-40 + 2^-30 of an edge (or outside FP32's range, or is not finite) and FP64 has to decide.
 __device__ __forceinline__ bool bin_fp32(float u, float v, float sh, float sl, float delta, int& bin) {
     if (u == 0.0f && v == 0.0f) {
         bin = 0;
