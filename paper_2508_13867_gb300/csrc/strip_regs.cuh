@@ -22,16 +22,16 @@
 // Work: the rows of the running samples, T samples side by side, are split into equal ranges, one per
 // group of G warps.  A piece (range x sample) of L rows runs L + 2 (NS - 1) iterations, so a batch with
 // fewer groups of samples than ranges splits each group into equal parts instead: no range then holds
-// parts of two (strip_part; 20 x 100^2 FP32: 2.8 us per step, equal ranges 4.1; 8 x
-// 256^2 3.6; 127^2 x 128 11.1, equal ranges 11.4).
+// parts of two (strip_part; 20 x 100^2 FP32: 2.8 us per step, equal ranges 4.1, both before idle lanes
+// loaded pairs of their own; 2.6 now).
 //
-// What bounds it (625 x 256^2 FP32, ncu): the register file's read ports.  A packed FMA of three
+// What bounds it (625 x 256^2 FP32): the register file's read ports and HBM.  A packed FMA of three
 // distinct registers takes three cycles (two with a reused or immediate operand, measured), about 600 of
-// the 830 cycles a warp's iteration takes; with loads and stores kept in cache the launch takes 0.50
-// instead of 0.53 ms.  HBM is at 0.85 of the copy bandwidth.  Against the strips with their rings in
-// shared memory, three steps per launch, two barriers per row: 126 against 168 us per step (324 against
-// 243 GLUPS); 128^2 319 / 242, 512^2 315 / 202, 1024^2 325 / 206, 255^2 271 / 210, 200^2 288 / 166; BF16 at
-// 256^2 294 / 235, FP16 280 / 231, FX16 227 / 217 (bound by its conversions).
+// the 800 cycles a warp's iteration takes; a launch of 0.498 ms moves its 2.95 GB at 0.87 of the copy
+// bandwidth.  Kernel GLUPS against the strips with their rings in shared memory, three steps per launch, two
+// barriers per row: 329 / 243 (125 against 168 us per step); 128^2 322 / 242, 512^2 329 / 202, 1024^2 325 / 206,
+// 255^2 277 / 210, 200^2 303 / 166; BF16 at 256^2 294 / 235, FP16 280 / 231, FX16 232 / 217 (bound by its
+// conversions).
 #pragma once
 
 // Number of phases (time steps) per launch.
@@ -255,7 +255,8 @@ __device__ __forceinline__ void strip_piece(const KParams& p, const StripPiece<S
             } else {
                 // FP32: the last two phases in scalar instructions (the same bits), which balances the
                 // register ports against the issue slots: 516 us per launch at 625 x 256^2, all packed
-                // 527, all scalar 529; 16-bit storage all packed 421, all scalar 449
+                // 527, all scalar 529 (an earlier build; 498 now); 16-bit storage all packed 421, all
+                // scalar 449
                 if (sizeof(S) == 4 && k >= 2)
                     collide_halves(h, om);
                 else
